@@ -21,6 +21,7 @@
 // (725 k FP64 multiply-adds per 21 x 21 footprint instead of 9.5 M).  The stamp
 // selection is exact: order statistics by radix selection on the values' bit
 // patterns, the MAD on the FP64 differences the definition takes.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include <algorithm>
@@ -29,62 +30,79 @@
 
 namespace ipp {
 
-// ---- stamp selection: one block per region ------------------------------------
-constexpr int SS_T = 1024, SS_W = SS_T / 32;
+// ---- stamp selection: one cluster of blocks per region ---------------------------
+// A region takes about 13 passes over its pixels (radix passes of the median and
+// the MAD, the extrema, the brightest pixel), and one block per region left SMs
+// idle and read the region from L2 each time.  Here NC <= 8 blocks of a cluster
+// share a region, each holds its slice in shared memory (84 KB; two blocks an SM)
+// and a pass ends in one exchange over distributed shared memory: the counters or
+// extrema of all blocks are read by every block, which then take the same decision.
+// Bound by the passes' integer work per element.  100 regions of 168 K pixels:
+// 820 -> 460 us.  A region above NC slices is read from memory in every pass.
+constexpr int SS_T = 512, SS_W = SS_T / 32, SS_NC = 8;
+constexpr int SS_SLICE = 21504;   // pixels of a slice: 84 KB beside 18 KB of counters, two blocks an SM
+
+struct StampShared {
+    unsigned int hist[SS_W * 256];
+    unsigned int tot[2][256];              // this block's digit counts, double-buffered over exchanges
+    unsigned long long xch[2][SS_NC];      // this block's values for an exchange
+    unsigned long long red[SS_NC][SS_W];
+    int sdig;
+    long long sbelow;
+};
 
 struct StampRegion {
     const float* I;
     const float* R;
     int64_t pitch, W, H;
     int x0, y0, rw, rh;   // the region [x0, x0 + rw) x [y0, y0 + rh)
-    int n;                // rw * rh
+    int t0, t1;           // this block's pixels of it (raster index)
+    bool cached;          // they are in shared memory
+    const float* cache;
+    int buf;              // exchange buffer in turn
 };
 
-__device__ __forceinline__ float reg_r(const StampRegion& g, int t, int* x, int* y) {
+__device__ __forceinline__ float reg_r(const StampRegion& g, int t) {
+    if (g.cached) return g.cache[t - g.t0];
     const int yy = t / g.rw;
-    *y = g.y0 + yy;
-    *x = g.x0 + (t - yy * g.rw);
-    return __ldg(g.R + (int64_t)*y * g.pitch + *x);
+    return __ldg(g.R + (int64_t)(g.y0 + yy) * g.pitch + (g.x0 + (t - yy * g.rw)));
 }
 
-// block sums / extrema (all threads call; result to all)
-__device__ long long block_sum_ll(long long v, long long* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    long long s = 0;
-    for (int w = 0; w < SS_W; w++) s += red[w];
-    __syncthreads();
-    return s;
+// One exchange: this block's value(s) in S.xch[buf] are combined over the
+// cluster's blocks by every block.  The buffers alternate, so one barrier per
+// exchange is enough: a buffer is written again only after the next barrier.
+__device__ __forceinline__ void stamp_barrier() { cooperative_groups::this_cluster().sync(); }
+
+template <class Op>
+__device__ __forceinline__ unsigned long long warp_red_u64(unsigned long long v, Op op) {
+    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
-__device__ unsigned long long block_max_u64(unsigned long long v, unsigned long long* red) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = t > v ? t : v;
+struct OpMin { __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a < b ? a : b; } };
+struct OpMax { __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a > b ? a : b; } };
+struct OpAdd { __device__ unsigned long long operator()(unsigned long long a, unsigned long long b) const { return a + b; } };
+
+// this block's partial of value `slot` (visible after the exchange's barrier)
+template <class Op>
+__device__ __forceinline__ void stamp_part(StampShared& S, int slot, unsigned long long v, Op op) {
+    v = warp_red_u64(v, op);
+    if ((threadIdx.x & 31) == 0) S.red[slot][threadIdx.x >> 5] = v;
+}
+template <class Op>
+__device__ __forceinline__ void stamp_block(StampShared& S, int buf, int slot, Op op) {   // after a block barrier
+    if (threadIdx.x == 0) {
+        unsigned long long v = S.red[slot][0];
+        for (int w = 1; w < SS_W; w++) v = op(v, S.red[slot][w]);
+        S.xch[buf][slot] = v;
     }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    unsigned long long m = 0;
-    for (int w = 0; w < SS_W; w++) m = red[w] > m ? red[w] : m;
-    __syncthreads();
-    return m;
 }
-
-__device__ unsigned long long block_min_u64(unsigned long long v, unsigned long long* red) {
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o);
-        v = t < v ? t : v;
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    unsigned long long m = ~0ull;
-    for (int w = 0; w < SS_W; w++) m = red[w] < m ? red[w] : m;
-    __syncthreads();
-    return m;
+template <class Op>
+__device__ __forceinline__ unsigned long long stamp_all(StampShared& S, int buf, int slot, Op op) {   // after the cluster barrier
+    auto cl = cooperative_groups::this_cluster();
+    unsigned long long v = *cl.map_shared_rank(&S.xch[buf][slot], 0);
+    for (unsigned r = 1; r < cl.num_blocks(); r++) v = op(v, *cl.map_shared_rank(&S.xch[buf][slot], r));
+    return v;
 }
 
 // Keys of a region's finite values for the order statistics, as unsigned
@@ -93,24 +111,25 @@ __device__ unsigned long long block_min_u64(unsigned long long v, unsigned long 
 //   mode 1: |v - med| exactly, as the integer |v 2^-e0 - med 2^-e0| -- every value
 //     and med are multiples of 2^e0 (e0: one below the smallest ulp in the
 //     region), so the difference is exact and its FP64 rounding is the FP64
-//     subtraction's, without the narrow FP64 pipe in the per-element work;
+//     subtraction's, without the narrow FP64 pipe in the per-element work; the
+//     scaling is two exact products with powers of two, 2^-e0 = s1 s2;
 //   mode 2: the bit pattern of the FP64 |v - med| (when the region's range does
 //     not fit 62 bits at scale 2^e0).
 struct KeySpec {
     int mode;
     int e0;
+    float s1, s2;
     double med;
     long long imed;
 };
 
 __device__ __forceinline__ bool stamp_key(const StampRegion& g, int t, const KeySpec& ks, unsigned long long* k) {
-    int x, y;
-    const float v = reg_r(g, t, &x, &y);
+    const float v = reg_r(g, t);
     if (!isfinite(v)) return false;
     if (ks.mode == 0) {
         *k = fkey(v);
     } else if (ks.mode == 1) {
-        const long long d = __float2ll_rz(ldexpf(v, -ks.e0)) - ks.imed;
+        const long long d = __float2ll_rz(__fmul_rn(__fmul_rn(v, ks.s1), ks.s2)) - ks.imed;
         *k = (unsigned long long)(d < 0 ? -d : d);
     } else {
         *k = (unsigned long long)__double_as_longlong(fabs((double)v - ks.med));
@@ -120,21 +139,21 @@ __device__ __forceinline__ bool stamp_key(const StampRegion& g, int t, const Key
 
 // The k-th smallest key (0-based) of the region: radix selection, 8 bits a
 // pass from bit top + 7 down, every key sharing the bits above top with
-// prefix0; per-warp histograms in shared memory (hist: SS_W x 256 counters),
-// fed by per-thread run lengths of equal digits.
-__device__ unsigned long long block_select(const StampRegion& g, const KeySpec& ks, long long k, int top,
-                                           unsigned long long prefix0, unsigned int* hist, int* sdig,
-                                           long long* sbelow) {
+// prefix0; per-warp histograms in shared memory, fed by per-thread run lengths
+// of equal digits, summed over the block, then over the cluster.
+__device__ unsigned long long region_select(StampRegion& g, const KeySpec& ks, long long k, int top,
+                                            unsigned long long prefix0, StampShared& S) {
+    auto cl = cooperative_groups::this_cluster();
     unsigned long long prefix = prefix0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int shift = top; shift >= 0; shift -= 8) {
-        for (int t = threadIdx.x; t < SS_W * 256; t += SS_T) hist[t] = 0;
+        for (int t = threadIdx.x; t < SS_W * 256; t += SS_T) S.hist[t] = 0;
         __syncthreads();
         // each thread counts runs of equal digits over its elements (the region's
         // keys mostly share their high digits) and adds a run to its warp's
         // histogram when the digit changes
         unsigned cur = 256u, run = 0u;
-        for (int t = threadIdx.x; t < g.n; t += SS_T) {
+        for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
             unsigned long long key = 0;
             bool ok = stamp_key(g, t, ks, &key);
             if (ok && shift + 8 < 64) ok = (key >> (shift + 8)) == prefix;
@@ -143,23 +162,30 @@ __device__ unsigned long long block_select(const StampRegion& g, const KeySpec& 
             if (dig == cur) {
                 run++;
             } else {
-                if (run) atomicAdd(&hist[warp * 256 + cur], run);
+                if (run) atomicAdd(&S.hist[warp * 256 + cur], run);
                 cur = dig;
                 run = 1u;
             }
         }
-        if (run) atomicAdd(&hist[warp * 256 + cur], run);
+        if (run) atomicAdd(&S.hist[warp * 256 + cur], run);
         __syncthreads();
-        // totals per digit (thread b < 256), then warp 0 finds the digit of rank k
         if (threadIdx.x < 256) {
             unsigned s = 0;
-            for (int w = 0; w < SS_W; w++) s += hist[w * 256 + threadIdx.x];
-            hist[threadIdx.x] = s;   // row 0 is no longer needed per warp
+            for (int w = 0; w < SS_W; w++) s += S.hist[w * 256 + threadIdx.x];
+            S.tot[g.buf][threadIdx.x] = s;
         }
+        cl.sync();
+        // the region's counts per digit (thread b < 256), then warp 0 finds the digit of rank k
+        if (threadIdx.x < 256) {
+            unsigned s = 0;
+            for (unsigned r = 0; r < cl.num_blocks(); r++) s += *cl.map_shared_rank(&S.tot[g.buf][threadIdx.x], r);
+            S.hist[threadIdx.x] = s;
+        }
+        g.buf ^= 1;
         __syncthreads();
         if (warp == 0) {
             long long c8 = 0;
-            for (int b = 0; b < 8; b++) c8 += hist[lane * 8 + b];
+            for (int b = 0; b < 8; b++) c8 += S.hist[lane * 8 + b];
             long long inc = c8;
             for (int o = 1; o < 32; o <<= 1) {
                 const long long u = __shfl_up_sync(0xffffffffu, inc, o);
@@ -171,53 +197,51 @@ __device__ unsigned long long block_select(const StampRegion& g, const KeySpec& 
                 long long c = exc;
                 int d = lane * 8;
                 for (int b = 0; b < 8; b++) {
-                    const long long nb = c + hist[lane * 8 + b];
+                    const long long nb = c + S.hist[lane * 8 + b];
                     if (k < nb) { d = lane * 8 + b; break; }
                     c = nb;
                 }
-                *sdig = d;
-                *sbelow = c;
+                S.sdig = d;
+                S.sbelow = c;
             }
         }
         __syncthreads();
-        prefix = (prefix << 8) | (unsigned long long)*sdig;
-        k -= *sbelow;
+        prefix = (prefix << 8) | (unsigned long long)S.sdig;
+        k -= S.sbelow;
         __syncthreads();
     }
     return prefix;
 }
 
-// (count of keys <= kk, smallest key > kk) over the region
-__device__ void block_count_next(const StampRegion& g, const KeySpec& ks, unsigned long long kk, long long* cnt,
-                                 unsigned long long* next, long long* red, unsigned long long* redu) {
-    long long c = 0;
-    unsigned long long nx = ~0ull;
-    for (int t = threadIdx.x; t < g.n; t += SS_T) {
-        unsigned long long key;
-        if (!stamp_key(g, t, ks, &key)) continue;
-        if (key <= kk) c++;
-        else if (key < nx) nx = key;
-    }
-    *cnt = block_sum_ll(c, red);
-    *next = block_min_u64(nx, redu);
-}
-
 // the two middle order statistics (k0 = (n - 1) / 2, k1 = n / 2) as keys, for
 // keys in [kmin, kmax]: the radix passes start at the highest byte where kmin
 // and kmax differ
-__device__ void block_middle(const StampRegion& g, const KeySpec& ks, long long n, unsigned long long kmin,
-                             unsigned long long kmax, unsigned int* hist, long long* red, unsigned long long* redu,
-                             int* sdig, long long* sbelow, unsigned long long* a, unsigned long long* b) {
+__device__ void region_middle(StampRegion& g, const KeySpec& ks, long long n, unsigned long long kmin,
+                              unsigned long long kmax, StampShared& S, unsigned long long* a, unsigned long long* b) {
     const long long k0 = (n - 1) / 2, k1 = n / 2;
     const unsigned long long dif = kmin ^ kmax;
     const int top = dif ? ((63 - __clzll((long long)dif)) & ~7) : 0;
     const unsigned long long prefix0 = top + 8 < 64 ? kmin >> (top + 8) : 0ull;
-    *a = block_select(g, ks, k0, top, prefix0, hist, sdig, sbelow);
+    *a = region_select(g, ks, k0, top, prefix0, S);
     if (k1 == k0) { *b = *a; return; }
-    long long cle;
-    unsigned long long nx;
-    block_count_next(g, ks, *a, &cle, &nx, red, redu);
-    *b = cle > k1 ? *a : nx;
+    // count of keys <= a, smallest key > a
+    unsigned long long c = 0, nx = ~0ull;
+    for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
+        unsigned long long key;
+        if (!stamp_key(g, t, ks, &key)) continue;
+        if (key <= *a) c++;
+        else if (key < nx) nx = key;
+    }
+    stamp_part(S, 0, c, OpAdd());
+    stamp_part(S, 1, nx, OpMin());
+    __syncthreads();
+    stamp_block(S, g.buf, 0, OpAdd());
+    stamp_block(S, g.buf, 1, OpMin());
+    stamp_barrier();
+    c = stamp_all(S, g.buf, 0, OpAdd());
+    nx = stamp_all(S, g.buf, 1, OpMin());
+    g.buf ^= 1;
+    *b = (long long)c > k1 ? *a : nx;
 }
 
 // Is every pixel of the (2 m + 1)^2 box of A around (x, y) finite?  (block-wide)
@@ -231,70 +255,92 @@ __device__ bool block_box_finite(const float* A, int64_t pitch, int x, int y, in
     return !__syncthreads_or(bad);
 }
 
-// One block per region: the candidate's pixel or -1.
-__global__ void __launch_bounds__(SS_T) k_sub_stamps(const float* I, const float* R, int64_t W, int64_t H,
-                                                     int64_t pitch, int nsx, int nsy, int hw, int fh, double nsig,
-                                                     int2* reg_out) {
-    __shared__ unsigned int hist[SS_W * 256];
-    __shared__ long long red[SS_W];
-    __shared__ unsigned long long redu[SS_W];
-    __shared__ int sdig;
-    __shared__ long long sbelow;
-    const int sx = blockIdx.x % nsx, sy = blockIdx.x / nsx;
+// One cluster per region: the candidate's pixel or -1.  Every block of the
+// cluster follows the same control flow on the same exchanged values.
+__global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const float* R, int64_t W, int64_t H,
+                                                        int64_t pitch, int nsx, int nsy, int hw, int fh, double nsig,
+                                                        int slice, int2* reg_out) {
+    extern __shared__ float stamp_cache[];   // [slice]
+    __shared__ StampShared S;
+    auto cl = cooperative_groups::this_cluster();
+    const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int reg = (int)blockIdx.x / nc;
+    const int sx = reg % nsx, sy = reg / nsx;
     StampRegion g;
     g.I = I; g.R = R; g.pitch = pitch; g.W = W; g.H = H;
     g.x0 = (int)(sx * W / nsx);
     g.y0 = (int)(sy * H / nsy);
     g.rw = (int)((sx + 1) * W / nsx) - g.x0;
     g.rh = (int)((sy + 1) * H / nsy) - g.y0;
-    g.n = g.rw * g.rh;
+    const int64_t npix = (int64_t)g.rw * g.rh;
+    g.t0 = (int)(npix * rank / nc);
+    g.t1 = (int)(npix * (rank + 1) / nc);
+    g.cached = false;
+    g.cache = stamp_cache;
+    g.buf = 0;
+    const bool fits = g.t1 - g.t0 <= slice;   // per block: no decision of the cluster depends on it
     // the finite values: count, key range, smallest ulp exponent, largest |v|
-    long long c = 0;
-    unsigned long long kmin = ~0ull, kmax = 0, emin = ~0ull, amax = 0;
-    for (int t = threadIdx.x; t < g.n; t += SS_T) {
-        int x, y;
-        const float v = reg_r(g, t, &x, &y);
+    uint32_t c = 0, kmin = ~0u, kmax = 0, emin = ~0u, amax = 0;
+    for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
+        const float v = reg_r(g, t);
+        if (fits) stamp_cache[t - g.t0] = v;
         if (!isfinite(v)) continue;
         c++;
-        const unsigned long long k = fkey(v);
-        kmin = k < kmin ? k : kmin;
-        kmax = k > kmax ? k : kmax;
-        const uint32_t bits = __float_as_uint(v) & 0x7fffffffu, be = bits >> 23;
-        const unsigned long long ue = be ? be : 1u;      // ulp 2^(be - 150), denormals as be = 1
-        emin = ue < emin ? ue : emin;
-        amax = bits > amax ? bits : amax;
+        const uint32_t k = fkey(v);
+        kmin = min(kmin, k);
+        kmax = max(kmax, k);
+        const uint32_t bits = __float_as_uint(v) & 0x7fffffffu;
+        emin = min(emin, max(bits >> 23, 1u));      // ulp 2^(be - 150), denormals as be = 1
+        amax = max(amax, bits);
     }
-    const long long n = block_sum_ll(c, red);
+    g.cached = fits;   // a thread reads back its own elements only
+    stamp_part(S, 0, c, OpAdd());
+    stamp_part(S, 1, kmin, OpMin());
+    stamp_part(S, 2, kmax, OpMax());
+    stamp_part(S, 3, emin, OpMin());
+    stamp_part(S, 4, amax, OpMax());
+    __syncthreads();
+    stamp_block(S, 0, 0, OpAdd());
+    stamp_block(S, 0, 1, OpMin());
+    stamp_block(S, 0, 2, OpMax());
+    stamp_block(S, 0, 3, OpMin());
+    stamp_block(S, 0, 4, OpMax());
+    stamp_barrier();
+    const long long n = (long long)stamp_all(S, 0, 0, OpAdd());
+    const unsigned long long gmin = stamp_all(S, 0, 1, OpMin()), gmax = stamp_all(S, 0, 2, OpMax());
+    emin = (uint32_t)stamp_all(S, 0, 3, OpMin());
+    amax = (uint32_t)stamp_all(S, 0, 4, OpMax());
+    g.buf = 1;
     if (n == 0) {
-        if (threadIdx.x == 0) reg_out[blockIdx.x] = make_int2(-1, -1);
+        if (rank == 0 && threadIdx.x == 0) reg_out[reg] = make_int2(-1, -1);
+        stamp_barrier();   // no block leaves while another reads its exchange buffer
         return;
     }
-    kmin = block_min_u64(kmin, redu);
-    kmax = block_max_u64(kmax, redu);
-    emin = block_min_u64(emin, redu);
-    amax = block_max_u64(amax, redu);
     // median (Eq. 1's even-count mean of the middle pair)
-    KeySpec ks{0, 0, 0.0, 0};
+    KeySpec ks{0, 0, 1.f, 1.f, 0.0, 0};
     unsigned long long ka, kb;
-    block_middle(g, ks, n, kmin, kmax, hist, red, redu, &sdig, &sbelow, &ka, &kb);
+    region_middle(g, ks, n, gmin, gmax, S, &ka, &kb);
     const double va = (double)fkey_inv((uint32_t)ka), vb = (double)fkey_inv((uint32_t)kb);
     const double med = (n & 1) ? vb : __dmul_rn(0.5, __dadd_rn(va, vb));
     // MAD: exact integer differences at scale 2^e0 when they fit 62 bits
     ks.med = med;
     ks.e0 = (int)emin - 150 - 1;
-    const double span = ldexp((double)__uint_as_float((uint32_t)amax) + fabs(med), -ks.e0);
+    const double span = ldexp((double)__uint_as_float(amax) + fabs(med), -ks.e0);
     double mad;
     if (span < 4.6e18) {
         ks.mode = 1;
+        // -150 <= e0 <= 103: two powers of two within the normal range, of one sign
+        const int h1 = -ks.e0 / 2, h2 = -ks.e0 - h1;
+        ks.s1 = __uint_as_float((uint32_t)(h1 + 127) << 23);
+        ks.s2 = __uint_as_float((uint32_t)(h2 + 127) << 23);
         ks.imed = __double2ll_rz(ldexp(med, -ks.e0));
-        const unsigned long long top =
-            (unsigned long long)ldexp((double)__uint_as_float((uint32_t)amax) + fabs(med), -ks.e0) + 1ull;
-        block_middle(g, ks, n, 0ull, top, hist, red, redu, &sdig, &sbelow, &ka, &kb);
+        const unsigned long long top = (unsigned long long)span + 1ull;
+        region_middle(g, ks, n, 0ull, top, S, &ka, &kb);
         const double da = ldexp((double)ka, ks.e0), db = ldexp((double)kb, ks.e0);
         mad = (n & 1) ? db : __dmul_rn(0.5, __dadd_rn(da, db));
     } else {
         ks.mode = 2;
-        block_middle(g, ks, n, 0ull, ~0ull, hist, red, redu, &sdig, &sbelow, &ka, &kb);
+        region_middle(g, ks, n, 0ull, ~0ull, S, &ka, &kb);
         const double da = __longlong_as_double((long long)ka), db = __longlong_as_double((long long)kb);
         mad = (n & 1) ? db : __dmul_rn(0.5, __dadd_rn(da, db));
     }
@@ -308,15 +354,23 @@ __global__ void __launch_bounds__(SS_T) k_sub_stamps(const float* I, const float
     float best = 0.f;
     for (;;) {
         unsigned long long mk = 0;
-        for (int t = threadIdx.x; t < g.n; t += SS_T) {
-            int x, y;
-            const float v = reg_r(g, t, &x, &y);
-            if (!isfinite(v) || x < m || y < m || x > W - 1 - m || y > H - 1 - m) continue;
+        for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
+            const float v = reg_r(g, t);
+            if (!isfinite(v)) continue;
+            const uint32_t fk = fkey(v);
+            if (fk < (uint32_t)(mk >> 32) || fk > (uint32_t)(bound >> 32)) continue;
+            const int yy = t / g.rw, y = g.y0 + yy, x = g.x0 + (t - yy * g.rw);
+            if (x < m || y < m || x > W - 1 - m || y > H - 1 - m) continue;
             const unsigned long long key =
-                ((unsigned long long)fkey(v) << 32) | (unsigned long long)(~(uint32_t)((int64_t)y * W + x));
+                ((unsigned long long)fk << 32) | (unsigned long long)(~(uint32_t)((int64_t)y * W + x));
             if (key < bound && key > mk) mk = key;
         }
-        mk = block_max_u64(mk, redu);
+        stamp_part(S, 0, mk, OpMax());
+        __syncthreads();
+        stamp_block(S, g.buf, 0, OpMax());
+        stamp_barrier();
+        mk = stamp_all(S, g.buf, 0, OpMax());
+        g.buf ^= 1;
         if (mk == 0) break;                              // no eligible pixel left
         const uint32_t idx = ~(uint32_t)(mk & 0xffffffffu);
         const int x = (int)(idx % (uint32_t)W), y = (int)(idx / (uint32_t)W);
@@ -327,8 +381,9 @@ __global__ void __launch_bounds__(SS_T) k_sub_stamps(const float* I, const float
         }
         bound = mk;
     }
-    if (threadIdx.x == 0)
-        reg_out[blockIdx.x] = (bx >= 0 && (double)best > thr) ? make_int2(bx, by) : make_int2(-1, -1);
+    if (rank == 0 && threadIdx.x == 0)
+        reg_out[reg] = (bx >= 0 && (double)best > thr) ? make_int2(bx, by) : make_int2(-1, -1);
+    stamp_barrier();   // no block leaves while another reads its exchange buffer
 }
 
 // Candidates in region order (row-major over the regions) and their count.
@@ -810,7 +865,32 @@ int ipp_launch_sub_stamps(const float* I, const float* R, int64_t W, int64_t H, 
                           int hw, int fh, double nsig, int32_t* cx, int32_t* cy, int32_t* n_dev, void* ws,
                           cudaStream_t s) {
     int2* reg = static_cast<int2*>(ws);   // the first array of the workspace
-    k_sub_stamps<<<(unsigned)(nsx * nsy), SS_T, 0, s>>>(I, R, W, H, pitch, nsx, nsy, hw, fh, nsig, reg);
+    // Blocks a region: as few as hold the largest region in their slices, then more
+    // while the grid stays within one wave of two blocks an SM and a slice keeps
+    // at least 8 pixels a thread (below that a pass is mostly its exchange).
+    const int64_t nreg = (int64_t)nsx * nsy, npix = ((W + nsx - 1) / nsx) * ((H + nsy - 1) / nsy);
+    int nc = 1;
+    while (nc < SS_NC && (npix > (int64_t)nc * SS_SLICE ||
+                          (nreg * nc * 2 <= 304 && npix >= (int64_t)nc * 2 * 8 * SS_T)))
+        nc *= 2;
+    const int slice = (int)std::min<int64_t>(SS_SLICE, npix / nc + 1);
+    auto fn = k_sub_stamps;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_SLICE * (int)sizeof(float)) !=
+        cudaSuccess)
+        return ipp_check_launch("k_sub_stamps shared memory");
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nreg * nc));
+    cfg.blockDim = dim3(SS_T);
+    cfg.dynamicSmemBytes = (size_t)slice * sizeof(float);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)nc;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, fn, I, R, W, H, pitch, nsx, nsy, hw, fh, nsig, slice, reg) != cudaSuccess)
+        return ipp_check_launch("k_sub_stamps");
     if (int e = ipp_check_launch("k_sub_stamps")) return e;
     k_sub_compact<<<1, 1024, 0, s>>>(reg, nsx * nsy, cx, cy, n_dev);
     return ipp_check_launch("k_sub_compact");
