@@ -457,22 +457,43 @@ __device__ void sub_terms_dev(double x, double y, int64_t W, int64_t H, int orde
     }
 }
 
-// one block per candidate: the footprint's C_n = R (x) K_n, separably
-__global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J) {
+// The footprint's C_n = R (x) K_n, separably.  FP64-bound (2 lanes a clock an SM:
+// one candidate's 725 K multiply-adds are 190 us of one SM), so a candidate is cut
+// into `parts` blocks that share nothing: block part takes the row filters
+// [f0, f1) -- a cut of about equal work -- and the basis functions built on them.
+// 100 candidates on 152 SMs: 200 -> 173 us with three parts each.
+__global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J, int parts) {
     extern __shared__ double sm[];
-    if ((int)blockIdx.x >= min(*J.n_dev, J.max_c)) return;
-    const int c = blockIdx.x;
+    const int c = blockIdx.x / parts, part = blockIdx.x - c * parts;
+    if (c >= min(*J.n_dev, J.max_c)) return;
     const int S = 2 * J.hw + 1, m = J.hw + J.fh, WS = 2 * m + 1, FW = 2 * J.fh + 1, nfp = FW * FW;
     double* h = sm;                    // [nf][S] one-dimensional filters
     double* Rw = h + J.nf * S;         // [WS][WS] the template around the candidate
     double* T = Rw + WS * WS;          // [nf][WS][FW] row-filtered template
     int2* bf = reinterpret_cast<int2*>(T + (size_t)J.nf * WS * FW);   // [nb] row and column filter of basis n
-    if (threadIdx.x == 0) {
-        int n = 0;
+    // row filters [f0, f1) and basis functions [n0, n1) of this part.  A filter's work:
+    // its rows (WS per footprint column) and, for each basis function on it, the
+    // footprint's columns (FW); it goes to the part that holds the middle of its share.
+    int f0 = -1, f1 = -1, n0 = 0, n1 = 0;
+    {
+        int total = 0, done = 0, n = 0;
         for (int k = 0; k < J.nk; k++)
-            for (int i = 0; i <= J.deg[k]; i++)
-                for (int j = 0; j <= J.deg[k] - i; j++) bf[n++] = make_int2(J.fo[k] + i, J.fo[k] + j);
+            for (int i = 0; i <= J.deg[k]; i++) total += WS + FW * (J.deg[k] - i + 1);
+        for (int k = 0; k < J.nk; k++)
+            for (int i = 0; i <= J.deg[k]; i++) {
+                const int nj = J.deg[k] - i + 1, w = WS + FW * nj;
+                if ((2 * done + w) * parts / (2 * total) == part) {
+                    if (f0 < 0) { f0 = J.fo[k] + i; n0 = n; }
+                    f1 = J.fo[k] + i + 1;
+                    n1 = n + nj;
+                }
+                done += w;
+                if (threadIdx.x == 0)
+                    for (int j = 0; j < nj; j++) bf[n + j] = make_int2(J.fo[k] + i, J.fo[k] + j);
+                n += nj;
+            }
     }
+    if (f0 < 0) return;
     for (int t = threadIdx.x; t < J.nf * S; t += 256) {
         const int f = t / S, u = t - f * S - J.hw;
         int k = 0;
@@ -491,7 +512,7 @@ __global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J) {
     }
     __syncthreads();
     // rows: T[f][r][q] = sum_u h_f(u) R(x - u, row r), x = footprint column q
-    for (int t = threadIdx.x; t < J.nf * WS * FW; t += 256) {
+    for (int t = f0 * WS * FW + threadIdx.x; t < f1 * WS * FW; t += 256) {
         const int f = t / (WS * FW), rq = t - f * WS * FW, r = rq / FW, q = rq - r * FW;
         const double* hf = h + f * S;
         const double* rr = Rw + r * WS + q + 2 * J.hw;   // R at column offset u = -hw .. hw: rr[-(u + hw)]
@@ -502,7 +523,7 @@ __global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J) {
     __syncthreads();
     // columns: C_n(p) = sum_v h_{k,j}(v) T_{k,i}(x, y - v)
     double* C = J.C + (size_t)c * J.nb * nfp;
-    for (int t = threadIdx.x; t < J.nb * nfp; t += 256) {
+    for (int t = n0 * nfp + threadIdx.x; t < n1 * nfp; t += 256) {
         const int n = t / nfp, p = t - n * nfp, pr = p / FW, pq = p - pr * FW;
         const int fi = bf[n].x, fj = bf[n].y;
         const double* hv = h + fj * S;
@@ -513,12 +534,14 @@ __global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J) {
     }
 }
 
-// one block per candidate: its Gram matrix of the C_n, the cross terms with the
-// background terms and the target, and the candidate's spatial terms
-__global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J) {
+// A candidate's Gram matrix of the C_n, the cross terms with the background terms
+// and the target, and the candidate's spatial terms.  FP64-bound as k_sub_conv, and
+// cut into `parts` blocks in the same way: each takes an equal run of
+// the sums.  100 candidates: 180 -> 138 us.
+__global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J, int parts) {
     extern __shared__ double sm[];
-    if ((int)blockIdx.x >= min(*J.n_dev, J.max_c)) return;
-    const int c = blockIdx.x;
+    const int c = blockIdx.x / parts, part = blockIdx.x - c * parts;
+    if (c >= min(*J.n_dev, J.max_c)) return;
     const int FW = 2 * J.fh + 1, nfp = FW * FW, nb = J.nb, ng = J.ng;
     double* Cs = sm;                   // [nb][nfp]
     double* Is = Cs + nb * nfp;        // [nfp]
@@ -537,7 +560,7 @@ __global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J) {
             for (int b = 0; b < ng; b++) Pb[b * nfp + p] = inb ? tb[b] : 0.0;
         }
     }
-    if (threadIdx.x == 0) {
+    if (part == 0 && threadIdx.x == 0) {
         double ts[64];
         sub_terms_dev((double)cx, (double)cy, J.W, J.H, J.sord, ts);
         for (int s = 0; s < J.ns; s++) J.Ps[(size_t)c * J.ns + s] = ts[s];
@@ -545,7 +568,8 @@ __global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J) {
     __syncthreads();
     const int ntri = nb * (nb + 1) / 2;
     const int ntask = ntri + nb * ng + nb + ng * ng + ng;
-    for (int t = threadIdx.x; t < ntask; t += 256) {
+    const int share = (ntask + parts - 1) / parts, tend = min(ntask, (part + 1) * share);
+    for (int t = part * share + threadIdx.x; t < tend; t += 256) {
         const double *a, *b;
         double* out;
         if (t < ntri) {                                   // G[n][m], m <= n
@@ -624,69 +648,105 @@ __global__ void __launch_bounds__(256) k_sub_assemble(SubFitJob J) {
 // panel of CB columns, the diagonal block is factored in shared memory
 // (k_chol_diag), the rows below it are solved against it (k_chol_trsm, a warp
 // per row), and the trailing lower triangle takes the panel's rank-CB update
-// (k_chol_syrk, a 32 x 32 tile per block).  Then the two triangular solves,
+// (k_chol_syrk, a tile per block).  Then the two triangular solves,
 // CB rows at a time (k_chol_solve).  FP64 throughout.  A pivot that is not
 // positive sets *status = 1; the later kernels then leave everything as is.
 constexpr int CB = 32;
 
 __global__ void k_chol_init(int32_t* status) { *status = 0; }
 
-__global__ void __launch_bounds__(256) k_chol_diag(double* A, int n, int k0, int32_t* status) {
+// The diagonal block.  Bound by the chain square root -> reciprocal -> scaled
+// column -> next pivot, so warp 0 runs that chain alone, one column ahead: it
+// brings column j + 1 up to date and factors it while the other warps apply column
+// j to the columns from j + 2 on; one barrier a column.  An entry still takes its
+// updates in ascending column order.  32 columns: 44 -> 28 us.
+constexpr int CD_T = 256, CD_W = CD_T / 32;
+
+__global__ void __launch_bounds__(CD_T) k_chol_diag(double* A, int n, int k0, int32_t* status) {
     __shared__ double D[CB][CB + 1];
-    __shared__ double rinv;
-    __shared__ int fail;
     if (__ldcg(status)) return;
-    const int b = min(CB, n - k0);
-    for (int t = threadIdx.x; t < b * b; t += 256) {
-        const int i = t / b, j = t - i * b;
-        D[i][j] = A[(size_t)(k0 + i) * n + k0 + j];
+    const int b = min(CB, n - k0), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int t = threadIdx.x; t < CB * CB; t += CD_T) {
+        const int i = t >> 5, j = t & 31;
+        D[i][j] = i < b && j <= i ? A[(size_t)(k0 + i) * n + k0 + j] : 0.0;
     }
-    if (threadIdx.x == 0) fail = 0;
     __syncthreads();
-    for (int j = 0; j < b; j++) {
-        if (threadIdx.x == 0) {
-            const double d = D[j][j];
-            if (!(d > 0.0)) fail = 1;
-            const double r = d > 0.0 ? sqrt(d) : 1.0;
-            D[j][j] = r;
-            rinv = 1.0 / r;
+    // column c, already up to date in lane i's v = D[i][c]: scaled by its pivot;
+    // returns whether the pivot is not positive
+    auto factor = [&](int c, double v) {
+        const double d = __shfl_sync(0xffffffffu, v, c);
+        const bool ok = d > 0.0;
+        const double r = ok ? sqrt(d) : 1.0;
+        const double rinv = 1.0 / r;
+        if (lane == c) D[lane][c] = r;
+        else if (lane > c) D[lane][c] = v * rinv;
+        return !ok;
+    };
+    bool bad = warp == 0 && factor(0, D[lane][0]);
+    bool fail = __syncthreads_or(bad);
+    for (int j = 0; j + 1 < b && !fail; j++) {
+        const double lj = lane > j ? D[lane][j] : 0.0;
+        if (warp == 0) {
+            const int c = j + 1;
+            double v = D[lane][c];
+            if (lane >= c) v -= lj * D[c][j];
+            bad = factor(c, v);
+        } else {
+            for (int c = j + 1 + warp; c < b; c += CD_W - 1) {
+                const double m = D[c][j];
+                if (lane >= c) D[lane][c] -= lj * m;
+            }
         }
-        __syncthreads();
-        if (fail) break;
-        for (int i = j + 1 + threadIdx.x; i < b; i += 256) D[i][j] *= rinv;
-        __syncthreads();
-        for (int t = threadIdx.x; t < b * b; t += 256) {          // trailing update inside the block
-            const int i = t / b, c = t - i * b;
-            if (i > j && c > j && c <= i) D[i][c] -= D[i][j] * D[c][j];
-        }
-        __syncthreads();
+        fail = __syncthreads_or(bad);
     }
     if (fail) {
         if (threadIdx.x == 0) *status = 1;
         return;
     }
-    for (int t = threadIdx.x; t < b * b; t += 256) {
-        const int i = t / b, j = t - i * b;
-        if (j <= i) A[(size_t)(k0 + i) * n + k0 + j] = D[i][j];
+    for (int t = threadIdx.x; t < CB * CB; t += CD_T) {
+        const int i = t >> 5, j = t & 31;
+        if (i < b && j <= i) A[(size_t)(k0 + i) * n + k0 + j] = D[i][j];
     }
 }
 
-// rows i >= k0 + CB: L21[i] = A21[i] L11^-T, one warp per row (lane j holds column j)
-__global__ void __launch_bounds__(256) k_chol_trsm(double* A, int n, int k0, const int32_t* status) {
+// a / b from y = RN(1 / b), correctly rounded (Markstein, IBM J. Res. Dev. 34,
+// 1990): the residual of a quotient within one ulp, formed exactly by an FMA, times
+// y corrects it to the rounded one.  The first product may be two ulps off, so the
+// correction is applied twice.  Outside the range in which no step can overflow or
+// lose bits the division itself.
+__device__ __forceinline__ double div_by_recip(double a, double b, double y) {
+    const double m = fabs(a);
+    if (m > 1e-200 && m < 1e200 && b > 1e-80 && b < 1e80) {
+        double q = a * y;
+        q = fma(fma(-q, b, a), y, q);
+        return fma(fma(-q, b, a), y, q);
+    }
+    return a / b;
+}
+
+// rows i >= k0 + CB: L21[i] = A21[i] L11^-T, one warp per row (lane j holds column
+// j).  A step is a quotient, a broadcast and a multiply-add; the quotients come from
+// the diagonal's reciprocals, taken once per block.  FP64 instructions of one SM
+// share a pipe of 2 lanes a clock, so two warps a block spread the rows over as many
+// SMs as there are.  265 rows: 23 -> 19 us (eight warps a block, a division a step).
+constexpr int CT_T = 64;
+
+__global__ void __launch_bounds__(CT_T) k_chol_trsm(double* A, int n, int k0, const int32_t* status) {
     __shared__ double L[CB][CB + 1];
     if (__ldcg(status)) return;
     const int b = min(CB, n - k0);
-    for (int t = threadIdx.x; t < b * b; t += 256) {
-        const int i = t / b, j = t - i * b;
-        L[i][j] = j <= i ? A[(size_t)(k0 + i) * n + k0 + j] : 0.0;
+    for (int t = threadIdx.x; t < CB * CB; t += CT_T) {
+        const int i = t >> 5, j = t & 31;
+        L[i][j] = i < b && j <= i ? A[(size_t)(k0 + i) * n + k0 + j] : (i == j ? 1.0 : 0.0);
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = k0 + b + blockIdx.x * 8 + warp; i < n; i += gridDim.x * 8) {
+    const double dl = L[lane][lane], yl = 1.0 / dl;
+    for (int i = k0 + b + blockIdx.x * (CT_T / 32) + warp; i < n; i += gridDim.x * (CT_T / 32)) {
         double a = lane < b ? A[(size_t)i * n + k0 + lane] : 0.0;
         double x = 0.0;
         for (int j = 0; j < b; j++) {
-            const double xj = __shfl_sync(0xffffffffu, lane == j ? a / L[j][j] : 0.0, j);
+            const double xj = __shfl_sync(0xffffffffu, lane == j ? div_by_recip(a, dl, yl) : 0.0, j);
             if (lane == j) x = xj;
             if (lane > j) a -= xj * L[lane][j];
         }
@@ -695,31 +755,34 @@ __global__ void __launch_bounds__(256) k_chol_trsm(double* A, int n, int k0, con
 }
 
 // trailing update of the lower triangle from row / column k0 + CB on: tile
-// (ti, tc), ti >= tc, of 32 x 32, A[i][c] -= sum_m L[i][k0 + m] L[c][k0 + m]
-__global__ void __launch_bounds__(256) k_chol_syrk(double* A, int n, int k0, const int32_t* status) {
-    __shared__ double Li[32][CB + 1], Lc[32][CB + 1];
+// (ti, tc), ti >= tc, of CS x CS, A[i][c] -= sum_m L[i][k0 + m] L[c][k0 + m].  Tiles
+// of 16 give every SM one at the first panels of ~300 unknowns (FP64-bound: 14 ->
+// 6 us with 32 x 32, which left two thirds of the SMs idle).
+constexpr int CS = 16;
+
+__global__ void __launch_bounds__(CS * CS) k_chol_syrk(double* A, int n, int k0, const int32_t* status) {
+    __shared__ double Li[CS][CB + 1], Lc[CS][CB + 1];
     if (__ldcg(status)) return;
     const int r0 = k0 + CB;
     const int t = blockIdx.x;
-    int ti = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+    int ti = (int)((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
     while (ti * (ti + 1) / 2 > t) ti--;
     while ((ti + 1) * (ti + 2) / 2 <= t) ti++;
     const int tc = t - ti * (ti + 1) / 2;
-    const int i0 = r0 + ti * 32, c0 = r0 + tc * 32;
-    for (int q = threadIdx.x; q < 32 * CB; q += 256) {
+    const int i0 = r0 + ti * CS, c0 = r0 + tc * CS;
+    for (int q = threadIdx.x; q < CS * CB; q += CS * CS) {
         const int r = q / CB, m = q - r * CB;
         Li[r][m] = i0 + r < n ? A[(size_t)(i0 + r) * n + k0 + m] : 0.0;
         Lc[r][m] = c0 + r < n ? A[(size_t)(c0 + r) * n + k0 + m] : 0.0;
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < 32 * 32; q += 256) {
-        const int r = q >> 5, c = q & 31;
-        const int i = i0 + r, cc = c0 + c;
-        if (i >= n || cc >= n || cc > i) continue;
-        double acc = 0.0;
-        for (int m = 0; m < CB; m++) acc = fma(Li[r][m], Lc[c][m], acc);
-        A[(size_t)i * n + cc] -= acc;
-    }
+    const int r = threadIdx.x / CS, c = threadIdx.x % CS;
+    const int i = i0 + r, cc = c0 + c;
+    if (i >= n || cc >= n || cc > i) return;
+    double acc = 0.0;
+#pragma unroll
+    for (int m = 0; m < CB; m++) acc = fma(Li[r][m], Lc[c][m], acc);
+    A[(size_t)i * n + cc] -= acc;
 }
 
 // L y = b, then L' x = y, CB rows at a time: the block's warps first take the
@@ -821,6 +884,19 @@ SubDims sub_dims(int hw, int fh, int nk, const int32_t* deg, int sord, int bord)
     return d;
 }
 
+// Blocks a candidate of the FP64-bound kernels, one block an SM: the cut whose
+// waves of 152 / parts candidates take the least time (100 candidates: one part
+// fills 100 SMs once, three fill 152 twice with a third of the work each).
+int sub_parts(int max_c) {
+    int best = 1;
+    double cost = 1e30;
+    for (int p = 1; p <= 6; p++) {
+        const double t = (double)(((int64_t)max_c * p + 151) / 152) / p;
+        if (t < cost * 0.95) { cost = t; best = p; }
+    }
+    return best;
+}
+
 // workspace: region results, then the per-candidate parts, the normal
 // equations and the candidate list of ipp_sub_fit
 size_t sub_carve(const SubDims& d, int max_c, int nreg, void* base, SubFitJob* J, int2** reg, int32_t** cxy) {
@@ -914,9 +990,10 @@ int ipp_launch_sub_normal(const float* I, const float* R, int64_t W, int64_t H, 
     if (max_c < 1) return IPP_OK;
     cudaFuncSetAttribute(k_sub_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.conv_smem);
     cudaFuncSetAttribute(k_sub_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.gram_smem);
-    k_sub_conv<<<(unsigned)max_c, 256, d.conv_smem, s>>>(J);
+    const int parts = sub_parts(max_c);
+    k_sub_conv<<<(unsigned)(max_c * parts), 256, d.conv_smem, s>>>(J, parts);
     if (int e = ipp_check_launch("k_sub_conv")) return e;
-    k_sub_gram<<<(unsigned)max_c, 256, d.gram_smem, s>>>(J);
+    k_sub_gram<<<(unsigned)(max_c * parts), 256, d.gram_smem, s>>>(J, parts);
     if (int e = ipp_check_launch("k_sub_gram")) return e;
     const int nt = d.np * (d.np + 1) / 2 + d.np;
     k_sub_assemble<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(J);
@@ -928,14 +1005,14 @@ int ipp_launch_sub_solve(double* AtA, double* Atb, int np, double* coef64, float
     k_chol_init<<<1, 1, 0, s>>>(status);
     if (int e = ipp_check_launch("k_chol_init")) return e;
     for (int k0 = 0; k0 < np; k0 += CB) {
-        k_chol_diag<<<1, 256, 0, s>>>(AtA, np, k0, status);
+        k_chol_diag<<<1, CD_T, 0, s>>>(AtA, np, k0, status);
         if (int e = ipp_check_launch("k_chol_diag")) return e;
         const int rest = np - k0 - CB;
         if (rest <= 0) break;
-        k_chol_trsm<<<(unsigned)std::min((rest + 7) / 8, 152), 256, 0, s>>>(AtA, np, k0, status);
+        k_chol_trsm<<<(unsigned)((rest + CT_T / 32 - 1) / (CT_T / 32)), CT_T, 0, s>>>(AtA, np, k0, status);
         if (int e = ipp_check_launch("k_chol_trsm")) return e;
-        const int nt = (rest + 31) / 32;
-        k_chol_syrk<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, s>>>(AtA, np, k0, status);
+        const int nt = (rest + CS - 1) / CS;
+        k_chol_syrk<<<(unsigned)(nt * (nt + 1) / 2), CS * CS, 0, s>>>(AtA, np, k0, status);
         if (int e = ipp_check_launch("k_chol_syrk")) return e;
     }
     k_chol_solve<<<1, 1024, 0, s>>>(AtA, Atb, np, coef64, coef, status);
