@@ -127,8 +127,7 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 // round:
 //   (1) idle slots take the next stamps of the chunk, in slot order; the warp
 //       stages each new stamp in shared memory (pixel k of slot s at
-//       k (32/G + 1) + s, so a column is written and a row read without bank
-//       conflicts) and computes its default starting point together;
+//       k fit_pitch(G) + s) and computes its default starting point together;
 //   (2) slots with a fit in progress solve their damped normal equations (FP64);
 //   (3) every slot with a point to try evaluates chi^2, J'WJ and J'Wr there,
 //       each lane of the slot over every G-th stamp row, and the slot's lanes
@@ -145,7 +144,33 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 // repeats every solve on both lanes of a slot, the FP64 pipe of this part
 // running at 1/64 of the FP32 rate.  Batches too small to give every lane a
 // stamp take G = 2 or 4 (fit_lanes_per_stamp), where the shorter rounds win.
+//
+// Bound by the latency of one lane's model evaluation with the two warps a scheduler
+// that the stamps' tiles leave room for, so at G = 1 a tile has no padding column
+// (15 x 15 stamps: 28.1 KB, eight warps an SM; 29 KB and seven before): a row, one
+// pixel of 32 stamps, is read without conflicts, and only the staging stores, one
+// stamp's column, meet in one bank.  200,000 stamps of 15 x 15: 15.3 -> 14.6 ms
+// with the forms of eval_lane and border_pair below.
 constexpr int FL_MAX_WARPS = 8;
+
+// Base-2 logarithm, exponential and quotient of the hardware without the steps that
+// extend them to subnormals: 1 + q >= 1 has none, and a profile value or derivative
+// below 2^-126 adds nothing to the sums.
+__device__ __forceinline__ float lg2_fast(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float ex2_fast(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float div_fast(float a, float b) {
+    float y;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
 
 // chi^2, J'WJ and J'Wr of one stamp at pp.  The model of psf_eval with the
 // per-trial constants (reciprocal widths, normalisation, trig) taken out of the
@@ -187,14 +212,14 @@ __device__ __forceinline__ float eval_lane(const float* __restrict__ col, const 
             const float q = fmaf(u, a, v * b);
             float A1, P, T;
             if (MODEL == IPP_PSF_GAUSS) {
-                A1 = A0 * exp2f(-0.72134752f * q);  // exp(-q/2)
+                A1 = A0 * ex2_fast(-0.72134752f * q);  // exp(-q/2)
                 P = F * A1;
                 T = -P;
             } else {
                 const float base = 1.0f + q;
-                A1 = A0 * exp2f(-beta * __log2f(base));
+                A1 = A0 * ex2_fast(-beta * lg2_fast(base));
                 P = F * A1;
-                T = __fdividef(tq * P, base);
+                T = div_fast(tq * P, base);
             }
             const float wk = WEIGHTED ? __ldg(wts + i * S + j) : 1.0f;
             const float r = row[j * PITCH] - (P + sky);
@@ -214,12 +239,16 @@ __device__ __forceinline__ float eval_lane(const float* __restrict__ col, const 
                 const float wa = wk * e[c];
                 gt[c] = fmaf(wa, r, gt[c]);
 #pragma unroll
-                for (int d = c; d < 7; d++) { Ht[t] = fmaf(wa, e[d], Ht[t]); t++; }
+                for (int d = c; d < 7; d++) {
+                    if (WEIGHTED || c != 3 || d != 3) Ht[t] = fmaf(wa, e[d], Ht[t]);
+                    t++;
+                }
             }
         }
         chi += rowc;
         star2 += rows;
     }
+    if (!WEIGHTED) Ht[18] = (float)((S - h + G - 1) / G * S);   // (sky, sky): the lane's pixels
     if (G > 1) {  // all lanes of the slot are here (their states are identical)
         const unsigned pm = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
 #pragma unroll
@@ -245,55 +274,73 @@ __device__ __forceinline__ int border_k(int b, int S) {
     return (1 + (c >> 1)) * S + ((c & 1) ? S - 1 : 0);
 }
 
-// Default start of stamp `sr` staged in column r: centre, border-median sky, sum
-// above sky, widths 1.6 / 1.4, theta 0.  All lanes of the warp take part and all
-// return the same values.  The border keys (at most 4 a lane for S <= 32) stay
-// in registers during the bisection for the two middle order statistics.
-template <int PITCH>
-__device__ __forceinline__ void init_coop(const float* __restrict__ sm, int r, int S, float p[7]) {
+// Order statistics k0 <= k1 of the border's keys, the same values in every lane.
+// Each lane holds at most 4 of the nb keys (S <= 32) and counts, for each, the keys
+// below and at most equal to it as every key passes by in a shuffle: the loads,
+// compares and shuffles are independent, where a bisection of the key range is 32
+// dependent rounds (0.6 against 2 K cycles of a warp for 15 x 15 stamps, with its
+// other lanes' fits waiting).
+template <int NK>
+__device__ __forceinline__ void border_pair(const uint32_t* key, int nb, int k0, int k1, uint32_t& ka, uint32_t& kb) {
+    const int lane = threadIdx.x & 31;
+    int lt[NK], le[NK];
+#pragma unroll
+    for (int s = 0; s < NK; s++) lt[s] = le[s] = 0;
+#pragma unroll
+    for (int t = 0; t < NK; t++) {
+        const int m = min(32, nb - 32 * t);
+#pragma unroll 8
+        for (int l = 0; l < m; l++) {
+            const uint32_t v = __shfl_sync(0xffffffffu, key[t], l);
+#pragma unroll
+            for (int s = 0; s < NK; s++) {
+                lt[s] += v < key[s];
+                le[s] += v <= key[s];
+            }
+        }
+    }
+    ka = kb = 0u;
+#pragma unroll
+    for (int s = 0; s < NK; s++) {
+        const bool mine = lane + 32 * s < nb;
+        const unsigned a = __ballot_sync(0xffffffffu, mine && lt[s] <= k0 && k0 < le[s]);
+        const unsigned b = __ballot_sync(0xffffffffu, mine && lt[s] <= k1 && k1 < le[s]);
+        if (a) ka = __shfl_sync(0xffffffffu, key[s], __ffs(a) - 1);
+        if (b) kb = __shfl_sync(0xffffffffu, key[s], __ffs(b) - 1);
+    }
+}
+
+// Default start of the stamp at src: centre, border-median sky, sum above sky,
+// widths 1.6 / 1.4, theta 0.  All lanes of the warp take part and all return the
+// same values.
+__device__ __forceinline__ void init_coop(const float* __restrict__ src, int S, float p[7]) {
     const int lane = threadIdx.x & 31;
     const int NP = S * S, nb = 4 * S - 4;
-    const int k0 = (nb - 1) / 2, k1 = nb / 2;
     uint32_t key[4];
 #pragma unroll
     for (int t = 0; t < 4; t++) {
         const int b = lane + 32 * t;
-        key[t] = b < nb ? fkey(sm[border_k(b, S) * PITCH + r]) : 0xffffffffu;
+        key[t] = b < nb ? fkey(__ldg(src + border_k(b, S))) : 0xffffffffu;
     }
-    const int nmine = (nb - lane + 31) >> 5;  // border values this lane holds
-    uint32_t lo = 0u, hi = 0xffffffffu;
-    while (lo < hi) {  // smallest key with more than k0 border values at or below it
-        const uint32_t mid = lo + ((hi - lo) >> 1);
-        int c = 0;
-#pragma unroll
-        for (int t = 0; t < 4; t++) c += t < nmine && key[t] <= mid;
-        c = warp_sum_i(c);
-        if (c > k0) hi = mid; else lo = mid + 1;
-    }
-    const uint32_t ka = lo;
-    int cle = 0;
-    uint32_t nxt = 0xffffffffu;
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-        if (t < nmine) {
-            cle += key[t] <= ka;
-            if (key[t] > ka && key[t] < nxt) nxt = key[t];
-        }
-    }
-    cle = warp_sum_i(cle);
-    nxt = __reduce_min_sync(0xffffffffu, nxt);
-    const uint32_t kb = cle > k1 ? ka : nxt;
+    uint32_t ka, kb;
+    if (nb <= 64) border_pair<2>(key, nb, (nb - 1) / 2, nb / 2, ka, kb);
+    else border_pair<4>(key, nb, (nb - 1) / 2, nb / 2, ka, kb);
     const float sky0 = (float)(0.5 * ((double)fkey_inv(ka) + (double)fkey_inv(kb)));
     float fs = 0.f;
-    for (int k = lane; k < NP; k += 32) fs += sm[k * PITCH + r] - sky0;
+    for (int k = lane; k < NP; k += 32) fs += __ldg(src + k) - sky0;
     fs = warp_sum(fs);
     p[0] = 0.5f * (S - 1); p[1] = 0.5f * (S - 1); p[2] = fs; p[3] = sky0;
     p[4] = 1.6f; p[5] = 1.4f; p[6] = 0.f;
 }
 
+constexpr int PF_AHEAD = 24;   // stamps
+
+// row pitch of a warp's tile: pixel k of slot s at k * pitch + s
+__host__ __device__ constexpr int fit_pitch(int G) { return G == 1 ? 32 : 32 / G + 1; }
+
 template <int MODEL, bool WEIGHTED, int G>
 __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t chunk) {
-    constexpr int SLOTS = 32 / G, PITCH = SLOTS + 1;
+    constexpr int PITCH = fit_pitch(G);
     extern __shared__ float fl_sm_all[];  // per warp [S*S][PITCH]: pixel k of slot s's stamp in column s
     __shared__ unsigned long long blk_next;  // next stamp of the block's chunk
     const unsigned FULL = 0xffffffffu;
@@ -341,6 +388,9 @@ __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t
                 nm &= nm - 1u;
                 const int64_t sr = __shfl_sync(FULL, st, rl);
                 const float* src = J.stamps + sr * NP;
+                // the stamp that a warp of the block will take about a round from now
+                if (sr + PF_AHEAD < c1 && lane * 32 < NP)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (int64_t)PF_AHEAD * NP + lane * 32));
                 for (int k = lane; k < NP; k += 32) fl_sm[k * PITCH + r] = __ldg(src + k);
                 __syncwarp();
                 if (J.init) {
@@ -350,7 +400,7 @@ __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t
                     }
                 } else {
                     float q[7];
-                    init_coop<PITCH>(fl_sm, r, S, q);
+                    init_coop(src, S, q);
                     if (slot == r) {
 #pragma unroll
                         for (int a = 0; a < 7; a++) p[a] = q[a];
@@ -606,9 +656,9 @@ static int sm_count() {
     return sms > 0 ? sms : 132;
 }
 
-static size_t fit_warp_bytes(int S, int G) { return (size_t)S * S * (32 / G + 1) * sizeof(float); }
-static int fit_max_warps(int S, int G) {
-    return (int)std::min<size_t>(FL_MAX_WARPS, (size_t)(227 * 1024) / fit_warp_bytes(S, G));
+static size_t fit_warp_bytes(int S, int G) { return (size_t)S * S * fit_pitch(G) * sizeof(float); }
+static int fit_max_warps(int S, int G) {   // the kernel's static shared memory is 8 bytes
+    return (int)std::min<size_t>(FL_MAX_WARPS, (size_t)(227 * 1024 - 64) / fit_warp_bytes(S, G));
 }
 
 template <int MODEL, bool WEIGHTED, int G>
@@ -637,10 +687,12 @@ static int launch_fit(const FitJob& J, cudaStream_t s) {
 // shorter.  G is taken while N G stays within 1.25 x the lanes resident at G
 // (measured on 152 SMs, 15 x 15 stamps: G = 4 up to ~12,000 stamps, G = 2 up
 // to ~24,000, G = 1 beyond).
+// G fixes the order of a stamp's sums, so the line does not move with the resident
+// warps of the present kernel: it counts eight warps at most.
 static int fit_lanes_per_stamp(const FitJob& J) {
     const int64_t sms = sm_count();
     for (int G = 4; G > 1; G >>= 1)
-        if (J.N * G * 4 <= sms * fit_max_warps(J.S, G) * 32 * 5) return G;
+        if (J.N * G * 4 <= sms * std::min(8, fit_max_warps(J.S, G)) * 32 * 5) return G;
     return 1;
 }
 
