@@ -15,7 +15,7 @@
 // multiply-adds costs C + 2 hw + 3 S / 4 shared loads: bound by the FP32 pipe
 // instead of shared memory.  Per output the sum still runs over the kernel's rows,
 // then columns, in ascending order.  4096 x 4096, hw = 10, 49 basis functions:
-// 767 -> 615 us (one row of 7 outputs a thread, before); the convolution's
+// 767 -> 532 us (one row of 7 outputs a thread, before); the convolution's
 // 7.4 G multiply-adds alone are 191 us of this part's FP32 rate.
 #include <math.h>
 
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
     constexpr int S = SH::S, T = SH::T, KP = SH::KP;
     __shared__ __align__(16) float Ks[TPB][S][KP];
     __shared__ float Rw[SH::WROWS * WP];   // the window, after the convolution its sums [S][TPB S]
-    __shared__ float an[TPB][SB_MAXB];
+    __shared__ __align__(16) float an[SB_MAXB][(TPB + 3) & ~3];
     const int ntx = (int)((W + S * TPB - 1) / (S * TPB));
     const int64_t bx = blockIdx.x % ntx, by = blockIdx.x / ntx;
     const int64_t x0 = bx * (S * TPB), y0 = by * S;
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
         const int ns = (sord + 1) * (sord + 2) / 2;
         float a = 0.f;
         for (int q = 0; q < ns; q++) a = fmaf(__ldg(cs + n * ns + q), P[q], a);
-        an[tile][n] = a;
+        an[n][tile] = a;
     }
     // template window: rows y0 - HW .., columns x0 - HW .. (0 outside the frame and
     // in the rows and columns that only padding outputs read)
@@ -123,21 +123,37 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
         Rw[a * WP + b] = in ? __ldg(R + yy * pitch + xx) : 0.f;
     }
     __syncthreads();
-    // Eq. 9 summed with the tiles' amplitudes: one read of a basis value serves the
-    // block's tiles
-    for (int t = threadIdx.x; t < S * S; t += T) {
-        float k[TPB];
+    // Eq. 9 summed with the tiles' amplitudes: one read of a basis value (from L2)
+    // serves the block's tiles, and the reads of all the thread's taps are in flight
+    {
+        constexpr int TAPS = (S * S + T - 1) / T;
+        float k[TAPS][TPB];
 #pragma unroll
-        for (int u = 0; u < TPB; u++) k[u] = 0.f;
-#pragma unroll 7
-        for (int n = 0; n < nb; n++) {
-            const float b = __ldg(basis + (size_t)n * S * S + t);
+        for (int m = 0; m < TAPS; m++)
 #pragma unroll
-            for (int u = 0; u < TPB; u++) k[u] = fmaf(an[u][n], b, k[u]);
+            for (int u = 0; u < TPB; u++) k[m][u] = 0.f;
+        const float* bp = basis + threadIdx.x;
+#pragma unroll 4
+        for (int n = 0; n < nb; n++, bp += S * S) {
+            float b[TAPS];
+#pragma unroll
+            for (int m = 0; m < TAPS; m++) b[m] = threadIdx.x + m * T < S * S ? __ldg(bp + m * T) : 0.f;
+#pragma unroll
+            for (int u = 0; u < TPB; u++) {
+                const float a = an[n][u];
+#pragma unroll
+                for (int m = 0; m < TAPS; m++) k[m][u] = fmaf(a, b[m], k[m][u]);
+            }
         }
-        const int vp = t / S, up = t - vp * S;
 #pragma unroll
-        for (int u = 0; u < TPB; u++) Ks[u][vp][up] = k[u];
+        for (int m = 0; m < TAPS; m++) {
+            const int t = threadIdx.x + m * T;
+            if (t < S * S) {
+                const int vp = t / S, up = t - vp * S;
+#pragma unroll
+                for (int u = 0; u < TPB; u++) Ks[u][vp][up] = k[m][u];
+            }
+        }
     }
     __syncthreads();
     const int tile = threadIdx.x / SH::TPT, rem = threadIdx.x - tile * SH::TPT;
