@@ -128,7 +128,9 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 //   (1) idle slots take the next stamps of the chunk, in slot order; the warp
 //       stages each new stamp in shared memory (pixel k of slot s at
 //       k fit_pitch(G) + s) and computes its default starting point together;
-//   (2) slots with a fit in progress solve their damped normal equations (FP64);
+//   (2) slots with a fit in progress solve their damped normal equations (FP64); one
+//       whose step promises little is put on hold until its convergence test, a
+//       second solve, can be made for several slots at once;
 //   (3) every slot with a point to try evaluates chi^2, J'WJ and J'Wr there,
 //       each lane of the slot over every G-th stamp row, and the slot's lanes
 //       add their sums with shuffles;
@@ -149,9 +151,16 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 // that the stamps' tiles leave room for, so at G = 1 a tile has no padding column
 // (15 x 15 stamps: 28.1 KB, eight warps an SM; 29 KB and seven before): a row, one
 // pixel of 32 stamps, is read without conflicts, and only the staging stores, one
-// stamp's column, meet in one bank.  200,000 stamps of 15 x 15: 15.3 -> 14.6 ms
+// stamp's column, meet in one bank.  200,000 stamps of 15 x 15: 15.3 -> 12.2 ms
 // with the forms of eval_lane and border_pair below.
 constexpr int FL_MAX_WARPS = 8;
+
+// Slots on hold for which the undamped system is solved (fewer when nothing else is
+// left to do in the warp).  A solve costs the warp the same FP64 time for one lane
+// as for 32, and with 32 fits a warp one of them converges in almost every round:
+// solved at once, the second solve doubled the FP64 work; waiting costs a slot a
+// round or two.
+constexpr int HOLD_MIN = 4;
 
 // Base-2 logarithm, exponential and quotient of the hardware without the steps that
 // extend them to subnormals: 1 + q >= 1 has none, and a profile value or derivative
@@ -289,7 +298,7 @@ __device__ __forceinline__ void border_pair(const uint32_t* key, int nb, int k0,
 #pragma unroll
     for (int t = 0; t < NK; t++) {
         const int m = min(32, nb - 32 * t);
-#pragma unroll 8
+#pragma unroll 4
         for (int l = 0; l < m; l++) {
             const uint32_t v = __shfl_sync(0xffffffffu, key[t], l);
 #pragma unroll
@@ -363,9 +372,10 @@ __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t
     float p[7], H[28], g[7], chi2 = 0.f, sm2 = 0.f;
     double lam = 0.0;
     int it = 0, nsing = 0;
-    bool fresh = false;
+    bool fresh = false, hold = false;
+    float pt[7];   // the point to try
 #pragma unroll
-    for (int a = 0; a < 7; a++) p[a] = 0.f;
+    for (int a = 0; a < 7; a++) p[a] = pt[a] = 0.f;
     while (true) {
         const unsigned idle = __ballot_sync(FULL, st < 0) & HEADS;
         if (idle && !drained) {
@@ -410,53 +420,59 @@ __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t
         }
         if (!__any_sync(FULL, st >= 0)) break;
 
-        float pt[7];
         bool try_pt = false;
         int fl = -1;
-        if (st >= 0) {
-            if (fresh) {
+        if (st >= 0 && fresh) {
 #pragma unroll
-                for (int a = 0; a < 7; a++) pt[a] = p[a];
-                try_pt = true;
+            for (int a = 0; a < 7; a++) pt[a] = p[a];
+            try_pt = true;
+        }
+        // pass 0: the damped step of every slot with a fit in progress; pass 1: the
+        // undamped system of the slots on hold.  One copy of the solve's code.
+#pragma unroll 1
+        for (int pass = 0; pass < 2; pass++) {
+            bool run = st >= 0 && !fresh && !hold;
+            if (pass == 1) {
+                const unsigned held = __ballot_sync(FULL, hold) & HEADS;
+                const bool due = __popc(held) >= HOLD_MIN / G || !__any_sync(FULL, try_pt);
+                run = hold && due;
+            }
+            if (!__any_sync(FULL, run)) continue;
+            if (!run) continue;
+            double x[7];
+            const bool ok = solve7(H, g, pass == 0 ? lam : 0.0, x);
+            if (!ok && pass == 0) {
+                lam *= 10.0;
+                nsing++;
+                it++;
+                if (lam > 1e10) fl = IPP_FLAG_FIT_MAXITER;
+                continue;
+            }
+            // converged when the Gauss-Newton decrease g'H^-1 g is below what the
+            // distance to the optimum (1e-10 chi^2) and the model's FP32 rounding
+            // (1e-12 sum w P^2) allow; the damped step's decrease never exceeds
+            // it, so the undamped system is solved only when that one is small
+            const double thr = 1e-10 * widen(chi2) + 1e-12 * widen(sm2);
+            double dec = 0.0;
+#pragma unroll
+            for (int a = 0; a < 7; a++) dec = fma(widen(g[a]), x[a], dec);
+            const bool small = ok && dec <= thr;
+            if (pass == 0) {
+#pragma unroll
+                for (int a = 0; a < 7; a++) pt[a] = narrow(widen(p[a]) + x[a]);
+                hold = small;
+                if (hold) continue;
             } else {
-                double delta[7];
-                if (!solve7(H, g, lam, delta)) {
-                    lam *= 10.0;
-                    nsing++;
-                    it++;
-                    if (lam > 1e10) fl = IPP_FLAG_FIT_MAXITER;
-                } else {
-                    {
-                        // converged when the Gauss-Newton decrease g'H^-1 g is below what the
-                        // distance to the optimum (1e-10 chi^2) and the model's FP32 rounding
-                        // (1e-12 sum w P^2) allow; the damped step's decrease never exceeds
-                        // it, so the undamped system is solved only when that one is small
-                        const double thr = 1e-10 * widen(chi2) + 1e-12 * widen(sm2);
-                        double dec = 0.0;
-#pragma unroll
-                        for (int a = 0; a < 7; a++) dec = fma(widen(g[a]), delta[a], dec);
-                        if (dec <= thr) {
-                            double dgn[7];
-                            if (solve7(H, g, 0.0, dgn)) {
-                                double dg = 0.0;
-#pragma unroll
-                                for (int a = 0; a < 7; a++) dg = fma(widen(g[a]), dgn[a], dg);
-                                if (dg <= thr) fl = 0;
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int a = 0; a < 7; a++) pt[a] = narrow(widen(p[a]) + delta[a]);
-                    if (fl == 0) {
-                        // stopped at p
-                    } else if (!(pt[4] > 0.05f) || !(pt[5] > 0.05f)) {
-                        lam *= 10.0;
-                        it++;
-                        if (lam > 1e10) fl = 0;
-                    } else {
-                        try_pt = true;
-                    }
-                }
+                hold = false;
+                if (small) fl = 0;   // stopped at p
+            }
+            if (fl == 0) {
+            } else if (!(pt[4] > 0.05f) || !(pt[5] > 0.05f)) {
+                lam *= 10.0;
+                it++;
+                if (lam > 1e10) fl = 0;
+            } else {
+                try_pt = true;
             }
         }
         float Ht[28], gt[7], c2t = 0.f, s2t = 0.f;
