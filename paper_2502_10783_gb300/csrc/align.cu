@@ -12,8 +12,8 @@
 // trigonometric call per node.  Then CD^-1 and Newton's method on the target's
 // SIP polynomial (at most 50 steps, stop below 1e-12 px; otherwise NaN).
 //
-// Reprojection: output pixel (j, i) samples the source at Minv (j, i, 1).  Each
-// warp takes 128 consecutive output pixels of a row: the segment's first source
+// Reprojection: output pixel (j, i) samples the source at Minv (j, i, 1).  A
+// warp task is 128 consecutive output pixels of a row: the segment's first source
 // position is formed in double-float arithmetic (FP32 pairs; the FP64 pipe of
 // this GPU is too narrow even for one FP64 evaluation per segment) and split
 // into an integer part and a fraction, and the lanes offset it in FP32
@@ -29,65 +29,65 @@ namespace ipp {
 constexpr int AL_T = 256;
 constexpr double AL_D2R = 3.14159265358979323846 / 180.0;
 
+// The two frames' WCS as the node loop uses them: the rotation and the target's
+// inverse CD matrix are formed on the host, once per call.
 struct WcsDev {
-    double crpix[2], crval[2], cd[4];
+    double crpix[2], cd[4];
     int a_order, b_order;
     double a[36], b[36];
 };
+struct WcsPair {
+    WcsDev src, tgt;
+    double R[9];      // target basis (east, north, centre) in the source basis
+    double icd[4];    // CD^-1 of the target, over one degree in radians
+};
 
+// SIP polynomial and its gradient by Horner's rule in u with coefficients that are
+// polynomials in v: two multiply-adds a term instead of the eight operations of
+// powers and products (this part's FP64 pipe bounds the node loop).
 __device__ __forceinline__ void sip_val_grad(const double* c, int order, double u, double v, double& f, double& fu,
                                              double& fv) {
-    double up[6], vp[6];
-    up[0] = vp[0] = 1.0;
-#pragma unroll
-    for (int k = 1; k < 6; k++) {
-        up[k] = up[k - 1] * u;
-        vp[k] = vp[k - 1] * v;
-    }
     f = fu = fv = 0.0;
     // fully unrolled: constant coefficient indices, terms above `order` skipped
 #pragma unroll
-    for (int p = 0; p < 6; p++) {
+    for (int p = 5; p >= 0; p--) {
+        if (p > order) continue;
+        double g = 0.0, gv = 0.0;   // sum_q c[p][q] v^q and its derivative
 #pragma unroll
-        for (int q = 0; q < 6 - p; q++) {
+        for (int q = 5 - p; q >= 0; q--) {
             if (p + q > order) continue;
-            const double k = c[p * 6 + q];
-            f += k * up[p] * vp[q];
-            if (p > 0) fu += k * p * up[p - 1] * vp[q];
-            if (q > 0) fv += k * q * up[p] * vp[q - 1];
+            gv = fma(gv, v, g);
+            g = fma(g, v, c[p * 6 + q]);
         }
+        fu = fma(fu, u, f);
+        f = fma(f, u, g);
+        fv = fma(fv, u, gv);
     }
 }
 
 __device__ __forceinline__ double sip_val(const double* c, int order, double u, double v) {
-    double f, fu, fv;
-    sip_val_grad(c, order, u, v, f, fu, fv);
+    double f = 0.0;
+#pragma unroll
+    for (int p = 5; p >= 0; p--) {
+        if (p > order) continue;
+        double g = 0.0;
+#pragma unroll
+        for (int q = 5 - p; q >= 0; q--) {
+            if (p + q > order) continue;
+            g = fma(g, v, c[p * 6 + q]);
+        }
+        f = fma(f, u, g);
+    }
     return f;
 }
 
-// target basis (east, north, centre) in the source basis: R[r][c] = t_r . s_c
-__device__ void wcs_rotation(const WcsDev& s, const WcsDev& t, double R[9]) {
-    double sa, ca, sd, cd, ta, tca, td, tcd;
-    sincos(s.crval[0] * AL_D2R, &sa, &ca);
-    sincos(s.crval[1] * AL_D2R, &sd, &cd);
-    sincos(t.crval[0] * AL_D2R, &ta, &tca);
-    sincos(t.crval[1] * AL_D2R, &td, &tcd);
-    const double S[3][3] = {{-sa, ca, 0.0}, {-sd * ca, -sd * sa, cd}, {cd * ca, cd * sa, sd}};      // e, n, c
-    const double T[3][3] = {{-ta, tca, 0.0}, {-td * tca, -td * ta, tcd}, {tcd * tca, tcd * ta, td}};
-    for (int r = 0; r < 3; r++)
-        for (int c = 0; c < 3; c++) R[r * 3 + c] = T[r][0] * S[c][0] + T[r][1] * S[c][1] + T[r][2] * S[c][2];
-}
-
-__global__ void __launch_bounds__(AL_T) k_wcs_map(WcsDev src, WcsDev tgt, int64_t nx, int64_t ny, int step,
+// Bound by FP64 (2 lanes a clock an SM).  128 x 128 nodes, SIP order 3: 31 -> 23 us
+// (the rotation's sines and cosines in every block, powers and products in the
+// polynomials and nine divisions a node and Newton step, before).
+__global__ void __launch_bounds__(AL_T) k_wcs_map(WcsPair P, int64_t nx, int64_t ny, int step,
                                                   double* __restrict__ xo, double* __restrict__ yo) {
-    __shared__ double R[9];
-    if (threadIdx.x < 32) {
-        double r[9];
-        wcs_rotation(src, tgt, r);
-        if (threadIdx.x < 9) R[threadIdx.x] = r[threadIdx.x];
-    }
-    __syncthreads();
-    const double det = tgt.cd[0] * tgt.cd[3] - tgt.cd[1] * tgt.cd[2];
+    const WcsDev &src = P.src, &tgt = P.tgt;
+    const double* R = P.R;
     const int64_t n = nx * ny;
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = k / nx, j = k - i * nx;
@@ -104,9 +104,10 @@ __global__ void __launch_bounds__(AL_T) k_wcs_map(WcsDev src, WcsDev tgt, int64_
         const double Z = R[6] * p + R[7] * q + R[8];
         double ox = NAN, oy = NAN;
         if (Z > 0.0) {
-            const double pt = X / Z / AL_D2R, qt = Y / Z / AL_D2R;
-            const double xt = (tgt.cd[3] * pt - tgt.cd[1] * qt) / det;
-            const double et = (-tgt.cd[2] * pt + tgt.cd[0] * qt) / det;
+            const double iz = 1.0 / Z;
+            const double pt = X * iz, qt = Y * iz;
+            const double xt = P.icd[0] * pt + P.icd[1] * qt;
+            const double et = P.icd[2] * pt + P.icd[3] * qt;
             double uu = xt, vv = et;
             bool ok = false;
             for (int it = 0; it < 50; it++) {
@@ -117,7 +118,8 @@ __global__ void __launch_bounds__(AL_T) k_wcs_map(WcsDev src, WcsDev tgt, int64_
                 const double j11 = 1.0 + fu, j12 = fv, j21 = gu, j22 = 1.0 + gv;
                 const double dj = j11 * j22 - j12 * j21;
                 if (dj == 0.0) break;
-                const double su = (j22 * r1 - j12 * r2) / dj, sv = (-j21 * r1 + j11 * r2) / dj;
+                const double id = 1.0 / dj;
+                const double su = (j22 * r1 - j12 * r2) * id, sv = (-j21 * r1 + j11 * r2) * id;
                 uu -= su;
                 vv -= sv;
                 if (fabs(su) < 1e-12 && fabs(sv) < 1e-12) {
@@ -136,7 +138,11 @@ __global__ void __launch_bounds__(AL_T) k_wcs_map(WcsDev src, WcsDev tgt, int64_
 }
 
 // ---- partial affine estimate -----------------------------------------------------
-constexpr int AF_BLOCKS = 152;
+// Two passes over the points (means, then centred moments); the last block of the
+// second pass to finish solves.  Latency- and FP64-bound: two warps a block keep the
+// butterflies short, the columns of partials are added and divided by one warp.
+// 16,384 points: 36 us in three launches -> 22 us in two.
+constexpr int AF_BLOCKS = 152, AF_SMALL = 64, AF_LARGE = 256;   // threads a block
 
 struct AffPts {
     const double *x, *y, *xt, *yt;
@@ -157,9 +163,10 @@ struct AffPts {
     }
 };
 
-// block sum of NV doubles in a fixed order (warp butterfly, then warps in order)
-template <int NV>
-__device__ void block_sum(double v[NV], double (*red)[AL_T / 32]) {
+// block sums of NV doubles in a fixed order (warp butterfly, then warps in order)
+// to out[0 .. NV), by the block's first threads
+template <int NV, int T>
+__device__ void block_sum(double v[NV], double (*red)[T / 32], double* out) {
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
 #pragma unroll
     for (int c = 0; c < NV; c++) {
@@ -168,20 +175,24 @@ __device__ void block_sum(double v[NV], double (*red)[AL_T / 32]) {
         if (lane == 0) red[c][wi] = v[c];
     }
     __syncthreads();
-#pragma unroll
-    for (int c = 0; c < NV; c++) {
+    if (threadIdx.x < NV) {
         double s = 0.0;
-        for (int k = 0; k < AL_T / 32; k++) s += red[c][k];
-        v[c] = s;
+        for (int k = 0; k < T / 32; k++) s += red[threadIdx.x][k];
+        out[threadIdx.x] = s;
     }
-    __syncthreads();
 }
 
+// Row of a block in the partials: 8 doubles, sums in the first five.  The sixth of
+// block 0's row in the first table counts the blocks of the second pass that are done.
+__device__ __forceinline__ unsigned int* aff_done(double* part1) { return reinterpret_cast<unsigned int*>(part1 + 5); }
+
 // pass 1: per-block count and coordinate sums
-__global__ void __launch_bounds__(AL_T) k_aff_sum1(AffPts P, double* __restrict__ part) {
-    __shared__ double red[5][AL_T / 32];
+template <int T>
+__global__ void __launch_bounds__(T) k_aff_sum1(AffPts P, double* __restrict__ part) {
+    __shared__ double red[5][T / 32];
     double v[5] = {0, 0, 0, 0, 0};
-    for (int64_t k = (int64_t)blockIdx.x * AL_T + threadIdx.x; k < P.n; k += (int64_t)gridDim.x * AL_T) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *aff_done(part) = 0u;
+    for (int64_t k = (int64_t)blockIdx.x * T + threadIdx.x; k < P.n; k += (int64_t)gridDim.x * T) {
         double a, b, c, d;
         if (!P.get(k, a, b, c, d)) continue;
         v[0] += 1.0;
@@ -190,8 +201,7 @@ __global__ void __launch_bounds__(AL_T) k_aff_sum1(AffPts P, double* __restrict_
         v[3] += c;
         v[4] += d;
     }
-    block_sum<5>(v, red);
-    if (threadIdx.x < 5) part[blockIdx.x * 8 + threadIdx.x] = v[threadIdx.x];
+    block_sum<5, T>(v, red, part + blockIdx.x * 8);
 }
 
 // sum of column q of the per-block partials, in the same order wherever it is
@@ -199,48 +209,15 @@ __global__ void __launch_bounds__(AL_T) k_aff_sum1(AffPts P, double* __restrict_
 __device__ __forceinline__ double aff_col(const double* part, int nb, int q) {
     const int lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += part[b * 8 + q];
+    for (int b = lane; b < nb; b += 32) s += __ldcg(part + b * 8 + q);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
 }
 
-// pass 2: per-block centred moments
-__global__ void __launch_bounds__(AL_T) k_aff_sum2(AffPts P, const double* __restrict__ part1,
-                                                   double* __restrict__ part2) {
-    __shared__ double red[3][AL_T / 32];
-    __shared__ double cs[5];
-    if (threadIdx.x < 32) {
-#pragma unroll
-        for (int q = 0; q < 5; q++) {
-            const double v = aff_col(part1, gridDim.x, q);
-            if (threadIdx.x == 0) cs[q] = v;
-        }
-    }
-    __syncthreads();
-    const double s[5] = {cs[0], cs[1], cs[2], cs[3], cs[4]};
-    const double m = s[0] > 0.0 ? s[0] : 1.0;
-    const double cx = s[1] / m, cy = s[2] / m, ctx = s[3] / m, cty = s[4] / m;
-    double v[3] = {0, 0, 0};
-    for (int64_t k = (int64_t)blockIdx.x * AL_T + threadIdx.x; k < P.n; k += (int64_t)gridDim.x * AL_T) {
-        double a, b, c, d;
-        if (!P.get(k, a, b, c, d)) continue;
-        const double dx = a - cx, dy = b - cy, ex = c - ctx, ey = d - cty;
-        v[0] += dx * dx + dy * dy;
-        v[1] += dx * ex + dy * ey;
-        v[2] += dx * ey - dy * ex;
-    }
-    block_sum<3>(v, red);
-    if (threadIdx.x < 3) part2[blockIdx.x * 8 + threadIdx.x] = v[threadIdx.x];
-}
-
-__global__ void k_aff_solve(const double* __restrict__ part1, const double* __restrict__ part2, int nb,
-                            double* __restrict__ M, int32_t* __restrict__ status) {
-    double s[5];
-#pragma unroll
-    for (int q = 0; q < 5; q++) s[q] = aff_col(part1, nb, q);
-    const double saa = aff_col(part2, nb, 0), sa = aff_col(part2, nb, 1), sb = aff_col(part2, nb, 2);
-    if (threadIdx.x != 0) return;
+// M and its inverse from the sums s (count, coordinates) and the centred moments
+__device__ void aff_solve(const double s[5], double saa, double sa, double sb, double* __restrict__ M,
+                          int32_t* __restrict__ status) {
     const double m = s[0];
     if (!(m >= 2.0) || !(saa > 0.0)) {
         for (int k = 0; k < 12; k++) M[k] = NAN;
@@ -264,7 +241,55 @@ __global__ void k_aff_solve(const double* __restrict__ part1, const double* __re
     if (status) *status = (s2 > 0.0) ? IPP_OK : IPP_ERR_DEGENERATE;
 }
 
+// pass 2: per-block centred moments; the last block to finish solves
+template <int T>
+__global__ void __launch_bounds__(T) k_aff_sum2(AffPts P, double* __restrict__ part1, double* __restrict__ part2,
+                                                   double* __restrict__ M, int32_t* __restrict__ status) {
+    __shared__ double red[3][T / 32];
+    __shared__ double cs[5], mean[4], mom[3];
+    __shared__ bool last;
+    const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int q = wi; q < 5; q += T / 32) {
+        const double v = aff_col(part1, gridDim.x, q);
+        if (lane == 0) cs[q] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) mean[threadIdx.x] = cs[threadIdx.x + 1] / (cs[0] > 0.0 ? cs[0] : 1.0);
+    __syncthreads();
+    const double cx = mean[0], cy = mean[1], ctx = mean[2], cty = mean[3];
+    double v[3] = {0, 0, 0};
+    for (int64_t k = (int64_t)blockIdx.x * T + threadIdx.x; k < P.n; k += (int64_t)gridDim.x * T) {
+        double a, b, c, d;
+        if (!P.get(k, a, b, c, d)) continue;
+        const double dx = a - cx, dy = b - cy, ex = c - ctx, ey = d - cty;
+        v[0] += dx * dx + dy * dy;
+        v[1] += dx * ex + dy * ey;
+        v[2] += dx * ey - dy * ex;
+    }
+    block_sum<3, T>(v, red, part2 + blockIdx.x * 8);
+    __threadfence();   // the partials before the count
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(aff_done(part1), 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int q = wi; q < 3; q += T / 32) {
+        const double t = aff_col(part2, gridDim.x, q);
+        if (lane == 0) mom[q] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double s[5] = {cs[0], cs[1], cs[2], cs[3], cs[4]};
+        aff_solve(s, mom[0], mom[1], mom[2], M, status);
+    }
+}
+
 // ---- bilinear reprojection ---------------------------------------------------------
+// A warp takes RP_GRP consecutive segments: its first lanes each form one segment's
+// double-float start, so that the ~250 instructions of a start are paid once per
+// group and not once per segment (they were half of the instructions of a segment's
+// 128 pixels).  4096 x 4096: 71 -> 54 us.
+constexpr int RP_GRP = 8;
 constexpr int RP_SEG = 128;   // output pixels per warp task (4 per lane)
 
 // df x exact float (|n| < 2^24): the product to ~2^-46 relative
@@ -347,8 +372,13 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ sr
     const int64_t warps = (int64_t)gridDim.x * (AL_T / 32);
     const float lim = 1073741824.f;   // 2^30: positions beyond are outside any frame
     const int Wi = (int)W, Hi = (int)H;
-    for (int64_t t = (int64_t)blockIdx.x * (AL_T / 32) + (threadIdx.x >> 5); t < tasks; t += warps) {
-        const int64_t i = t / segs, j0 = (t - i * segs) * RP_SEG;
+    for (int64_t t0 = ((int64_t)blockIdx.x * (AL_T / 32) + (threadIdx.x >> 5)) * RP_GRP; t0 < tasks;
+         t0 += warps * RP_GRP) {
+      // lane l: segment t0 + l's row, first column and source position
+      int mi = 0, mj = 0, mbx = 0, mby = 0, mok = 0;
+      float mfx = 0.f, mfy = 0.f;
+      if (lane < RP_GRP && t0 + lane < tasks) {
+        const int64_t i = (t0 + lane) / segs, j0 = (t0 + lane - i * segs) * RP_SEG;
         // first source position of the segment, Minv (j0, i, 1), in double-float
         const float fj = (float)(int)j0, fi = (float)(int)i;   // exact: Wo, Ho < 2^24
         const df X0 = df_add(df_add(df_mul_exact(m0, fj), df_mul_exact(m1, fi)), m2);
@@ -371,6 +401,17 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ sr
             const int iya = iby + (int)floorf(fby), iyb = iby + (int)floorf(yb);
             interior = min(ixa, ixb) >= 0 && max(ixa, ixb) <= Wi - 2 && min(iya, iyb) >= 0 && max(iya, iyb) <= Hi - 2;
         }
+        mi = (int)i; mj = (int)j0; mbx = ibx; mby = iby; mfx = fbx; mfy = fby;
+        mok = (base_ok ? 1 : 0) | (interior ? 2 : 0);
+      }
+      const int nseg = (int)min((int64_t)RP_GRP, tasks - t0);
+      for (int g = 0; g < nseg; g++) {
+        const int64_t i = __shfl_sync(0xffffffffu, mi, g), j0 = __shfl_sync(0xffffffffu, mj, g);
+        const int ibx = __shfl_sync(0xffffffffu, mbx, g), iby = __shfl_sync(0xffffffffu, mby, g);
+        const float fbx = __shfl_sync(0xffffffffu, mfx, g), fby = __shfl_sync(0xffffffffu, mfy, g);
+        const int ok = __shfl_sync(0xffffffffu, mok, g);
+        const bool base_ok = ok & 1, interior = ok & 2;
+        const int kmax = (int)min((int64_t)RP_SEG, Wo - j0) - 1;
         float v[4];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
@@ -406,6 +447,7 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ sr
             for (int c = 0; c < 4; c++)
                 if (jj + c < Wo) orow[jj + c] = v[c];
         }
+      }
     }
 }
 
@@ -423,10 +465,7 @@ static unsigned al_grid(int64_t units_per_block_task, int64_t tasks, int per_sm)
 
 static WcsDev to_dev(const ipp_wcs& w) {
     WcsDev d;
-    for (int k = 0; k < 2; k++) {
-        d.crpix[k] = w.crpix[k];
-        d.crval[k] = w.crval[k];
-    }
+    for (int k = 0; k < 2; k++) d.crpix[k] = w.crpix[k];
     for (int k = 0; k < 4; k++) d.cd[k] = w.cd[k];
     d.a_order = w.a_order;
     d.b_order = w.b_order;
@@ -437,10 +476,31 @@ static WcsDev to_dev(const ipp_wcs& w) {
     return d;
 }
 
+// target basis (east, north, centre) in the source basis: R[r][c] = t_r . s_c
+static void wcs_rotation(const ipp_wcs& s, const ipp_wcs& t, double R[9]) {
+    const double sa = sin(s.crval[0] * AL_D2R), ca = cos(s.crval[0] * AL_D2R);
+    const double sd = sin(s.crval[1] * AL_D2R), cd = cos(s.crval[1] * AL_D2R);
+    const double ta = sin(t.crval[0] * AL_D2R), tca = cos(t.crval[0] * AL_D2R);
+    const double td = sin(t.crval[1] * AL_D2R), tcd = cos(t.crval[1] * AL_D2R);
+    const double S[3][3] = {{-sa, ca, 0.0}, {-sd * ca, -sd * sa, cd}, {cd * ca, cd * sa, sd}};      // e, n, c
+    const double T[3][3] = {{-ta, tca, 0.0}, {-td * tca, -td * ta, tcd}, {tcd * tca, tcd * ta, td}};
+    for (int r = 0; r < 3; r++)
+        for (int c = 0; c < 3; c++) R[r * 3 + c] = T[r][0] * S[c][0] + T[r][1] * S[c][1] + T[r][2] * S[c][2];
+}
+
 int ipp_launch_wcs_map(const ipp_wcs& src, const ipp_wcs& tgt, int64_t nx, int64_t ny, int step, double* xo,
                        double* yo, cudaStream_t s) {
+    WcsPair P;
+    P.src = to_dev(src);
+    P.tgt = to_dev(tgt);
+    wcs_rotation(src, tgt, P.R);
+    const double k = 1.0 / ((tgt.cd[0] * tgt.cd[3] - tgt.cd[1] * tgt.cd[2]) * AL_D2R);
+    P.icd[0] = tgt.cd[3] * k;
+    P.icd[1] = -tgt.cd[1] * k;
+    P.icd[2] = -tgt.cd[2] * k;
+    P.icd[3] = tgt.cd[0] * k;
     // FP64-bound: 64-thread blocks so that small node grids still reach every SM
-    k_wcs_map<<<al_grid(64, nx * ny, 16), 64, 0, s>>>(to_dev(src), to_dev(tgt), nx, ny, step, xo, yo);
+    k_wcs_map<<<al_grid(64, nx * ny, 16), 64, 0, s>>>(P, nx, ny, step, xo, yo);
     return ipp_check_launch("k_wcs_map");
 }
 
@@ -451,19 +511,25 @@ int ipp_launch_affine_fit(const double* x, const double* y, const double* xt, co
     AffPts P{x, y, xt, yt, n, grid_nx, step};
     double* p1 = (double*)ws;
     double* p2 = p1 + AF_BLOCKS * 8;
-    k_aff_sum1<<<AF_BLOCKS, AL_T, 0, s>>>(P, p1);
-    if (int e = ipp_check_launch("k_aff_sum1")) return e;
-    k_aff_sum2<<<AF_BLOCKS, AL_T, 0, s>>>(P, p1, p2);
-    if (int e = ipp_check_launch("k_aff_sum2")) return e;
-    k_aff_solve<<<1, 32, 0, s>>>(p1, p2, AF_BLOCKS, M, status);
-    return ipp_check_launch("k_aff_solve");
+    // two warps a block while a thread has at most eight points; beyond that the
+    // loads of eight warps are wanted in flight
+    if (n <= (int64_t)8 * AF_BLOCKS * AF_SMALL) {
+        k_aff_sum1<AF_SMALL><<<AF_BLOCKS, AF_SMALL, 0, s>>>(P, p1);
+        if (int e = ipp_check_launch("k_aff_sum1")) return e;
+        k_aff_sum2<AF_SMALL><<<AF_BLOCKS, AF_SMALL, 0, s>>>(P, p1, p2, M, status);
+    } else {
+        k_aff_sum1<AF_LARGE><<<AF_BLOCKS, AF_LARGE, 0, s>>>(P, p1);
+        if (int e = ipp_check_launch("k_aff_sum1")) return e;
+        k_aff_sum2<AF_LARGE><<<AF_BLOCKS, AF_LARGE, 0, s>>>(P, p1, p2, M, status);
+    }
+    return ipp_check_launch("k_aff_sum2");
 }
 
 int ipp_launch_reproject(const float* src, int64_t W, int64_t H, int64_t pitch, const double* Minv, int64_t Wo,
                          int64_t Ho, float fill, float* out, int64_t opitch, cudaStream_t s) {
     const bool vout = (opitch % 4 == 0) && (((uintptr_t)out & 15) == 0);
     const int64_t tasks = ((Wo + RP_SEG - 1) / RP_SEG) * Ho;
-    k_reproject<<<al_grid(AL_T / 32, tasks, 8), AL_T, 0, s>>>(src, W, H, pitch, Minv, Wo, Ho, fill, out, opitch,
-                                                               vout);
+    k_reproject<<<al_grid(AL_T / 32 * RP_GRP, tasks, 8), AL_T, 0, s>>>(src, W, H, pitch, Minv, Wo, Ho, fill, out, opitch,
+                                                                        vout);
     return ipp_check_launch("k_reproject");
 }
