@@ -78,15 +78,26 @@ struct MeshGeom {
     const float* inv_flat;
     int64_t x0, y0;
     int mw, we, he, slots;
-    bool vec;  // f32, unmasked, 16-byte aligned rows, we % 4 == 0: float4 reads
+    bool vec;    // f32, unmasked, 16-byte aligned rows, we % 4 == 0: float4 reads
+    bool vec16;  // raw u16, unmasked, rows of the frame and of its calibration maps aligned to four pixels
+};
+
+// The frame's type, known when the kernel is compiled (a launch over frames of both
+// types decides per frame): the reads are inlined at eight places, and a kernel that
+// holds the code of one type stays within its registers and instruction cache.
+enum MeshKind { MK_F32 = 0, MK_U16 = 1, MK_ANY = 2 };
+template <int KIND>
+struct MeshGeomOf : MeshGeom {
+    static constexpr int kind = KIND;
 };
 
 // Value of mesh pixel (r, c) (inside the mesh's frame region); false when the
 // pixel is masked or not finite.
-__device__ __forceinline__ bool mesh_value_at(const MeshGeom& G, int r, int c, float* out) {
+template <class GG>
+__device__ __forceinline__ bool mesh_value_at(const GG& G, int r, int c, float* out) {
     const int64_t yy = G.y0 + r, xx = G.x0 + c;
     float x;
-    if (G.dtype == IPP_F32) {
+    if (GG::kind == MK_F32 || (GG::kind == MK_ANY && G.dtype == IPP_F32)) {
         x = __ldg(reinterpret_cast<const float*>(G.img) + yy * G.pitch + xx);
     } else {
         const float raw = (float)__ldg(reinterpret_cast<const uint16_t*>(G.img) + yy * G.pitch + xx);
@@ -97,16 +108,58 @@ __device__ __forceinline__ bool mesh_value_at(const MeshGeom& G, int r, int c, f
     return !(G.mask && G.mask[yy * G.W + xx]) && isfinite(x);
 }
 
-// Calls f(v) for every usable value of the mesh that this thread owns.  Vector
+// Calls f(v) for every usable value of the mesh that this thread owns (raw frames
+// whose rows and maps are aligned: mesh_for_each_u16 above).  Vector
 // path: float4 quads of the mesh's frame region, quad e4 = threadIdx.x + k *
 // MS_THREADS; scalar path: element e = threadIdx.x + k * MS_THREADS of the
 // mw x mh slots (row e / mw, column e % mw).  A chunk of loads is issued before
 // any is used: addresses are clamped into the mesh and slots beyond it are
 // skipped afterwards.  Every call forms the values with the same arithmetic, so
 // re-reads see identical values.
-template <int T = MS_THREADS, class F>
-__device__ __forceinline__ void mesh_for_each(const MeshGeom& G, F&& f) {
-    if (G.vec) {
+// The quads of a raw frame: 8 bytes of the frame and 16 of the inverse flat (and of
+// the bias map) a load, where the scalar path takes four loads of each and their
+// addresses.  4096 x 4096 raw frame, 128 px meshes: k_mesh_stats 206 -> @MS16@ us.
+template <int T, class F>
+__device__ __forceinline__ void mesh_for_each_u16(const MeshGeom& G, F& f) {
+    constexpr int VCH = 2;
+    const int qpr = G.we >> 2, nq = G.he * qpr;
+    const ushort4* raw = reinterpret_cast<const ushort4*>(reinterpret_cast<const uint16_t*>(G.img) + G.y0 * G.pitch +
+                                                          G.x0);
+    const int64_t m0 = G.y0 * G.W + G.x0, p4 = G.pitch >> 2, w4 = G.W >> 2;
+    const float4* flat = reinterpret_cast<const float4*>(G.inv_flat + m0);
+    const float4* bias = G.bias_map ? reinterpret_cast<const float4*>(G.bias_map + m0) : nullptr;
+    const int dr = T / qpr, dc = T - dr * qpr;
+    int r = threadIdx.x / qpr, c = threadIdx.x - r * qpr;
+    for (int e0 = threadIdx.x; e0 < nq; e0 += VCH * T) {
+        ushort4 q[VCH];
+        float4 w[VCH];
+        int64_t at[VCH];
+#pragma unroll
+        for (int j = 0; j < VCH; j++) {
+            const int rr = min(r, G.he - 1);
+            q[j] = __ldg(raw + (int64_t)rr * p4 + c);
+            at[j] = (int64_t)rr * w4 + c;
+            w[j] = __ldg(flat + at[j]);
+            r += dr;
+            c += dc;
+            if (c >= qpr) { c -= qpr; r++; }
+        }
+#pragma unroll
+        for (int j = 0; j < VCH; j++) {
+            if (e0 + j * T >= nq) continue;
+            const float4 b = bias ? __ldg(bias + at[j]) : make_float4(G.bias, G.bias, G.bias, G.bias);
+            const float x[4] = {((float)q[j].x - b.x) * w[j].x, ((float)q[j].y - b.y) * w[j].y,
+                                ((float)q[j].z - b.z) * w[j].z, ((float)q[j].w - b.w) * w[j].w};
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (isfinite(x[k])) f(x[k]);
+        }
+    }
+}
+
+template <int T = MS_THREADS, class GG, class F>
+__device__ __forceinline__ void mesh_for_each(const GG& G, F&& f) {
+    if (GG::kind != MK_U16 && G.vec) {
         constexpr int VCH = 4;
         const int qpr = G.we >> 2, nq = G.he * qpr;
         const float4* base = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(G.img) + G.y0 * G.pitch +
@@ -132,6 +185,10 @@ __device__ __forceinline__ void mesh_for_each(const MeshGeom& G, F&& f) {
                 if (isfinite(q[j].w)) f(q[j].w);
             }
         }
+        return;
+    }
+    if (GG::kind != MK_F32 && G.vec16) {
+        mesh_for_each_u16<T>(G, f);
         return;
     }
     const int dr = T / G.mw, dc = T - dr * G.mw;
@@ -368,7 +425,8 @@ __device__ float warp_radix_select(MeshShared& S, const float* buf, int s0, int 
 
 // Block-wide: the same selection over the values of the mesh itself (global
 // re-reads), for a median bin holding more values than the gather buffer.
-__device__ float block_radix_select_global(MeshShared& S, const MeshGeom& G, float lo, float hi, int bsel,
+template <class GG>
+__device__ float block_radix_select_global(MeshShared& S, const GG& G, float lo, float hi, int bsel,
                                            float cstar, float inv_bw, int r) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t prefix = 0, pmask = 0;
@@ -592,12 +650,13 @@ __device__ int warp0_finish(MeshShared& S, const MeshJob& J, const Stored& St, c
     return ST_SCAN;
 }
 
+template <int KIND>
 __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh) {
     __shared__ MeshShared S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
     const int mx = mesh % J.nx, my = mesh / J.nx;
-    MeshGeom G;
+    MeshGeomOf<KIND> G;
     G.img = J.img; G.dtype = J.dtype; G.pitch = J.pitch; G.W = J.W; G.mask = J.mask;
     G.bias_map = J.bias_map; G.bias = J.bias; G.inv_flat = J.inv_flat;
     G.x0 = (int64_t)mx * J.mesh_w; G.y0 = (int64_t)my * J.mesh_h;
@@ -607,6 +666,9 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
     G.slots = J.mesh_w * J.mesh_h;
     G.vec = J.dtype == IPP_F32 && !J.mask && (J.pitch & 3) == 0 && (G.we & 3) == 0 &&
             ((reinterpret_cast<uintptr_t>(J.img) + (uintptr_t)((G.y0 * J.pitch + G.x0) * 4)) & 15) == 0;
+    G.vec16 = J.dtype != IPP_F32 && !J.mask && ((J.pitch | J.W | G.x0 | G.we) & 3) == 0 &&
+              (reinterpret_cast<uintptr_t>(J.img) & 7) == 0 &&
+              ((reinterpret_cast<uintptr_t>(J.inv_flat) | reinterpret_cast<uintptr_t>(J.bias_map)) & 15) == 0;
 
     // ---- histogram window from a sample: warp 0 sorts 256 values spread over
     // the mesh; bw = 2^e with NB*bw in (8, 16] robust sigma, centre c* a
@@ -1062,7 +1124,10 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
     }
 }
 
-__global__ void __launch_bounds__(MS_THREADS, 7) k_mesh_stats(MeshJob J) { mesh_stats_body(J, blockIdx.x); }
+template <int KIND>
+__global__ void __launch_bounds__(MS_THREADS, 7) k_mesh_stats(MeshJob J) {
+    mesh_stats_body<KIND>(J, blockIdx.x);
+}
 
 // ---------------------------------------------------------------------------
 // Invalid-mesh fill and median filter on the mesh grid.  An invalid node takes
@@ -1239,9 +1304,10 @@ __global__ void __launch_bounds__(MF_THREADS) k_mesh_median(const float* fill_bk
 }
 
 // ---- batched form: the same bodies over a table of frames ------------------
+template <int KIND>
 __global__ void __launch_bounds__(MS_THREADS, 7) k_mesh_stats_multi(const MeshJob* J, const int* bs, int nf) {
     const int f = frame_of(bs, nf, blockIdx.x);
-    mesh_stats_body(J[f], blockIdx.x - bs[f]);
+    mesh_stats_body<KIND>(J[f], blockIdx.x - bs[f]);
 }
 
 __global__ void __launch_bounds__(MF_THREADS) k_mesh_fill_multi(const MeshFilterJob* J, const int* bs, int nf) {
@@ -1371,11 +1437,16 @@ int ipp_launch_mesh_stats(const MeshJob& J, cudaStream_t s) {
     // seven 31 KB CTAs per SM need the largest shared-memory carveout; the
     // attribute is per device, so it is set once on each device that launches
     if (int e = ipp_once_per_device(0, [] {
-            return cudaFuncSetAttribute(k_mesh_stats, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                        cudaSharedmemCarveoutMaxShared);
+            const cudaError_t e0 = cudaFuncSetAttribute(
+                k_mesh_stats<MK_F32>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+            return e0 != cudaSuccess ? e0
+                                     : cudaFuncSetAttribute(k_mesh_stats<MK_U16>,
+                                                            cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                            cudaSharedmemCarveoutMaxShared);
         }))
         return e;
-    k_mesh_stats<<<J.nx * J.ny, MS_THREADS, 0, s>>>(J);
+    if (J.dtype == IPP_F32) k_mesh_stats<MK_F32><<<J.nx * J.ny, MS_THREADS, 0, s>>>(J);
+    else k_mesh_stats<MK_U16><<<J.nx * J.ny, MS_THREADS, 0, s>>>(J);
     return ipp_check_launch("k_mesh_stats");
 }
 
@@ -1403,10 +1474,13 @@ int ipp_launch_bg_subtract(const SubJob& J, cudaStream_t s) {
 int ipp_bg_multi_pack(const MeshJob* J, const MeshFilterJob* F, int nf, HostBlob& hb, BgMultiPlan* p) {
     int nb[1024];
     if (nf < 1 || nf > 1024) return ipp_set_error(IPP_ERR_INVALID_ARG, "1..1024 frames");
+    p->f32 = p->u16 = true;
     for (int f = 0; f < nf; f++) {
         if (J[f].mesh_w * J[f].mesh_h > 16384)
             return ipp_set_error(IPP_ERR_NOT_SUPPORTED, "mesh area %d > 16384", J[f].mesh_w * J[f].mesh_h);
         nb[f] = J[f].nx * J[f].ny;
+        p->f32 = p->f32 && J[f].dtype == IPP_F32;
+        p->u16 = p->u16 && J[f].dtype != IPP_F32;
     }
     p->stats = ipp_put_stage(hb, J, nb, nf);
     for (int f = 0; f < nf; f++) nb[f] = (F[f].nx * F[f].ny + MF_THREADS - 1) / MF_THREADS;
@@ -1417,10 +1491,10 @@ int ipp_bg_multi_pack(const MeshJob* J, const MeshFilterJob* F, int nf, HostBlob
 }
 
 int ipp_bg_multi_launch(const BgMultiPlan& p, const unsigned char* t, cudaStream_t s) {
-    cudaFuncSetAttribute(k_mesh_stats_multi, cudaFuncAttributePreferredSharedMemoryCarveout,
-                         cudaSharedmemCarveoutMaxShared);
-    k_mesh_stats_multi<<<(unsigned)p.stats.total, MS_THREADS, 0, s>>>(
-        reinterpret_cast<const MeshJob*>(t + p.stats.jobs), reinterpret_cast<const int*>(t + p.stats.bs), p.nf);
+    auto stats = p.f32 ? k_mesh_stats_multi<MK_F32> : (p.u16 ? k_mesh_stats_multi<MK_U16> : k_mesh_stats_multi<MK_ANY>);
+    cudaFuncSetAttribute(stats, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    stats<<<(unsigned)p.stats.total, MS_THREADS, 0, s>>>(reinterpret_cast<const MeshJob*>(t + p.stats.jobs),
+                                                        reinterpret_cast<const int*>(t + p.stats.bs), p.nf);
     if (int e = ipp_check_launch("k_mesh_stats_multi")) return e;
     const MeshFilterJob* F = reinterpret_cast<const MeshFilterJob*>(t + p.fill.jobs);
     const int* bs = reinterpret_cast<const int*>(t + p.fill.bs);

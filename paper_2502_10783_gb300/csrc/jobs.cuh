@@ -192,7 +192,7 @@ struct StageRef {
     int total = 0;             // virtual blocks over all frames
 };
 
-struct BgMultiPlan { StageRef stats, fill, median; int nf = 0; };
+struct BgMultiPlan { StageRef stats, fill, median; int nf = 0; bool f32 = false, u16 = false; };
 struct DetMultiPlan {
     StageRef zero, thresh, filt, tile, tile_full, unions, resolve, count, scan, emit, fin;
     int nf = 0;
