@@ -199,7 +199,7 @@ struct DetMultiPlan {
     bool poly = true, filter = false;
     size_t scan_smem = 0;
 };
-struct PhotMultiPlan { StageRef cen, ap; int nf = 0; size_t ap_smem = 0; };
+struct PhotMultiPlan { StageRef cen, ap; int nf = 0; size_t ap_smem = 0; bool cen_small = false; };
 }  // namespace ipp
 
 template <class T>
