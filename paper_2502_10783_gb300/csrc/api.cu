@@ -1,5 +1,6 @@
 // api.cu -- the C ABI of libipp: argument validation, workspace layout and the
 // launch sequences of each call.  All calls are asynchronous on `stream`.
+#include <atomic>
 #include <stdarg.h>
 #include <mutex>
 #include <cmath>
@@ -42,6 +43,17 @@ int ipp_once_per_device_impl(int slot, cudaError_t (*fn)(void*), void* arg) {
     if (e != cudaSuccess) return ipp_set_error(IPP_ERR_CUDA, "per-device set-up: %s", cudaGetErrorString(e));
     g_once_done[dev] |= (uint16_t)(1u << slot);
     return IPP_OK;
+}
+
+int ipp_sm_count() {
+    static std::atomic<int> count[64];
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && (n = count[dev].load(std::memory_order_relaxed)) > 0) return n;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) return 152;
+    if (dev >= 0 && dev < 64) count[dev].store(n, std::memory_order_relaxed);
+    return n;
 }
 
 extern "C" const char* ipp_status_string(int status) {

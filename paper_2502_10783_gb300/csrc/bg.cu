@@ -1126,6 +1126,7 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
 
 template <int KIND>
 __global__ void __launch_bounds__(MS_THREADS, 7) k_mesh_stats(MeshJob J) {
+    dep_begin();
     mesh_stats_body<KIND>(J, blockIdx.x);
 }
 
@@ -1285,6 +1286,7 @@ __device__ __forceinline__ void mesh_fill_body(const float* raw_bkg, const float
 
 __global__ void __launch_bounds__(MF_THREADS) k_mesh_fill(const float* raw_bkg, const float* raw_rms, int nx, int ny,
                                                           float* fill_bkg, float* fill_rms, int32_t* status_dev) {
+    dep_begin();
     mesh_fill_body(raw_bkg, raw_rms, nx, ny, fill_bkg, fill_rms, status_dev, blockIdx.x);
 }
 
@@ -1300,6 +1302,7 @@ __device__ __forceinline__ void mesh_median_body(const float* fill_bkg, const fl
 
 __global__ void __launch_bounds__(MF_THREADS) k_mesh_median(const float* fill_bkg, const float* fill_rms, int nx,
                                                             int ny, int fw, int fh, float* out_bkg, float* out_rms) {
+    dep_begin();
     mesh_median_body(fill_bkg, fill_rms, nx, ny, fw, fh, out_bkg, out_rms, blockIdx.x);
 }
 
@@ -1445,8 +1448,8 @@ int ipp_launch_mesh_stats(const MeshJob& J, cudaStream_t s) {
                                                             cudaSharedmemCarveoutMaxShared);
         }))
         return e;
-    if (J.dtype == IPP_F32) k_mesh_stats<MK_F32><<<J.nx * J.ny, MS_THREADS, 0, s>>>(J);
-    else k_mesh_stats<MK_U16><<<J.nx * J.ny, MS_THREADS, 0, s>>>(J);
+    ipp_launch_dep(J.dtype == IPP_F32 ? k_mesh_stats<MK_F32> : k_mesh_stats<MK_U16>, dim3(J.nx * J.ny), MS_THREADS, 0,
+                   s, J);
     return ipp_check_launch("k_mesh_stats");
 }
 
@@ -1456,9 +1459,9 @@ int ipp_launch_mesh_filter(const float* raw_bkg, const float* raw_rms, float* fi
     const int nn = nx * ny;
     if (!fill_bkg || !fill_rms) return ipp_set_error(IPP_ERR_INVALID_ARG, "fill arrays NULL");
     const int blocks = (nn + MF_THREADS - 1) / MF_THREADS;
-    k_mesh_fill<<<blocks, MF_THREADS, 0, s>>>(raw_bkg, raw_rms, nx, ny, fill_bkg, fill_rms, status_dev);
+    ipp_launch_dep(k_mesh_fill, dim3(blocks), MF_THREADS, 0, s, raw_bkg, raw_rms, nx, ny, fill_bkg, fill_rms, status_dev);
     if (int e = ipp_check_launch("k_mesh_fill")) return e;
-    k_mesh_median<<<blocks, MF_THREADS, 0, s>>>(fill_bkg, fill_rms, nx, ny, fw, fh, out_bkg, out_rms);
+    ipp_launch_dep(k_mesh_median, dim3(blocks), MF_THREADS, 0, s, fill_bkg, fill_rms, nx, ny, fw, fh, out_bkg, out_rms);
     return ipp_check_launch("k_mesh_median");
 }
 

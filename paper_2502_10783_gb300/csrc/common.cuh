@@ -110,11 +110,15 @@ IPP_D df df_from_i64(long long i) {
 // v - c 2^-8 (|.| <= 2^-9, formed exactly in FP32) in units of 2^-40.  Sums of
 // such pairs are exact and order-independent; the c sums stay in range while
 // the totals stay below ~3.6e16 (values, or values times pixel coordinates).
+// Conversions to and from 32-bit integers: the 64-bit ones go through this part's
+// narrow FP64 pipe (15% of k_tile_label's time); |v| 2^8 at or above 2^31 takes them.
 IPP_D void fx_split(float v, long long out[2]) {
-    const long long c = __float2ll_rn(v * 256.0f);
-    const float rsd = fabsf(v) < 65536.0f ? v - (float)c * (1.0f / 256.0f) : 0.0f;
-    out[0] = c;
-    out[1] = __float2ll_rn(rsd * 1099511627776.0f);
+    const float a = v * 256.0f;
+    out[0] = fabsf(a) < 2147483648.0f ? (long long)__float2int_rn(a) : __float2ll_rn(a);
+    const float rsd = fabsf(v) < 65536.0f ? v - rintf(a) * (1.0f / 256.0f) : 0.0f;
+    // |rsd| 2^40 <= 2^31; the conversion saturates at 2^31 - 1, a float only as 2^31
+    const int f = __float2int_rn(rsd * 1099511627776.0f);
+    out[1] = f == 0x7fffffff ? 2147483648LL : (long long)f;
 }
 // the pair's value in double-float
 IPP_D df fx_value(const long long* p) {
@@ -151,6 +155,17 @@ IPP_D int frame_of(const int* bs, int nf, int b) {
     return lo;
 }
 
+// Programmatic dependent launch.  The kernels of a frame's chain start with
+// dep_begin(): nothing of the earlier kernels is touched before they are complete
+// and visible, and a grid small enough to leave room lets the next kernel's blocks
+// take their places meanwhile, so that a small frame's 14 launches do not each pay
+// the drain and the start of a grid.  Larger grids, whose waiting successors would
+// hold places that other streams' kernels could use, leave that to their end.
+IPP_D void dep_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (gridDim.x * gridDim.y <= 608u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 IPP_HD int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 IPP_HD int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
@@ -159,6 +174,27 @@ IPP_HD int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 // host-side error recording (api.cu)
 int ipp_set_error(int status, const char* fmt, ...);
 int ipp_check_launch(const char* what);
+
+// Launch of a kernel that starts with dep_begin(): its blocks may be placed before
+// the previous kernel of the stream is complete.  A failed launch is left as the
+// runtime's last error (ipp_check_launch).
+template <class... P, class... A>
+void ipp_launch_dep(void (*k)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, static_cast<A&&>(args)...);
+}
+
+// Number of SMs of the current device (queried once per device).
+int ipp_sm_count();
 
 // Runs fn() (a host callable returning cudaError_t) once per (slot, device) for
 // the current device, under a lock; later calls return at once.  For per-device

@@ -81,7 +81,14 @@ struct SubThreshJob {
     bool filter;                      // threshold the 3 x 3 pyramid-smoothed sub (not fused)
     uint32_t* mask;                   // [H][mw] bit rows, bit b of word w = column 32 w + b
     int64_t mw;
+    int32_t* zero;                    // words that block 0 clears for the labeling passes (NULL: none)
+    int nzero;
 };
+
+__device__ __forceinline__ void thresh_clear(const SubThreshJob& J) {
+    if (J.zero && blockIdx.x == 0 && blockIdx.y == 0)
+        for (int t = threadIdx.x; t < J.nzero; t += blockDim.x) J.zero[t] = 0;
+}
 
 struct TileJob {
     int64_t W, H;
@@ -361,6 +368,8 @@ __device__ __forceinline__ void sub_thresh_body(const SubThreshJob& J, int bx, i
 }
 
 __global__ void __launch_bounds__(ST_THREADS, 4) k_sub_thresh(SubThreshJob J) {
+    dep_begin();
+    thresh_clear(J);
     sub_thresh_body(J, blockIdx.x, blockIdx.y);
 }
 
@@ -522,6 +531,8 @@ __device__ __forceinline__ void sub_thresh_poly_body(const SubThreshJob& J, int 
 }
 
 __global__ void __launch_bounds__(ST_THREADS, 4) k_sub_thresh_poly(SubThreshJob J) {
+    dep_begin();
+    thresh_clear(J);
     sub_thresh_poly_body(J, blockIdx.x, blockIdx.y);
 }
 
@@ -730,7 +741,10 @@ __device__ __forceinline__ void tile_label_fast(const TileJob& J, int tile) {
     }
 }
 
-__global__ void __launch_bounds__(T_THREADS) k_tile_label(TileJob J) { tile_label_fast(J, blockIdx.y * J.ntx + blockIdx.x); }
+__global__ void __launch_bounds__(T_THREADS) k_tile_label(TileJob J) {
+    dep_begin();
+    tile_label_fast(J, blockIdx.y * J.ntx + blockIdx.x);
+}
 
 // Full pass over the listed tiles (any mask fits: T_RCAP is the most runs a
 // tile can have).
@@ -741,7 +755,10 @@ __device__ __forceinline__ void tile_label_full(const TileJob& J, int vb, int nv
     for (int i = vb; i < n; i += nvb) tile_label_body(J, S, __ldcg(J.ws.ovf + i));
 }
 
-__global__ void __launch_bounds__(T_THREADS) k_tile_label_full(TileJob J) { tile_label_full(J, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(T_THREADS) k_tile_label_full(TileJob J) {
+    dep_begin();
+    tile_label_full(J, blockIdx.x, gridDim.x);
+}
 
 // ------------------------------------------------------------ global phase
 __device__ __forceinline__ int gfind(int32_t* P, int x) {
@@ -1001,10 +1018,12 @@ __device__ void ccl_final_tile(const CclWs& ws, int32_t* lab, int tile, int64_t 
 // which needs all its blocks resident at once, stops the labeling of one frame
 // from overlapping the kernels of frames on other streams.)
 __global__ void __launch_bounds__(G_THREADS) k_ccl_union(CclWs ws, int ntx, int nty) {
+    dep_begin();
     ccl_union_tile(ws, blockIdx.x, ntx, nty);
 }
 
 __global__ void __launch_bounds__(G_THREADS) k_ccl_resolve(CclWs ws) {
+    dep_begin();
     const int n = __ldcg(ws.counters);
     for (int t = blockIdx.x * G_THREADS + threadIdx.x; t < n; t += gridDim.x * G_THREADS)
         ccl_resolve_node(ws, __ldcg(ws.klist + t));
@@ -1012,16 +1031,19 @@ __global__ void __launch_bounds__(G_THREADS) k_ccl_resolve(CclWs ws) {
 
 __global__ void __launch_bounds__(G_THREADS) k_ccl_count(CclWs ws, int64_t W, int ntx, int min_area) {
     __shared__ GShared G;
+    dep_begin();
     ccl_count_tile(ws, G, blockIdx.x, W, ntx, min_area);
 }
 
 __global__ void __launch_bounds__(G_THREADS) k_ccl_scan(CclWs ws, int ntx, int nty, int32_t* n_src_dev) {
     extern __shared__ __align__(16) int g_sm[];   // 2 T_TH ntx ints
     __shared__ GShared G;
+    dep_begin();
     ccl_scan_row(ws, G, g_sm, blockIdx.x, ntx, nty, n_src_dev);
 }
 
 __global__ void __launch_bounds__(G_THREADS) k_ccl_emit(CclWs ws, int32_t max_src, ipp_src_stats out) {
+    dep_begin();
     const int n = __ldcg(ws.counters);
     for (int t = blockIdx.x * G_THREADS + threadIdx.x; t < n; t += gridDim.x * G_THREADS)
         ccl_emit_node(ws, __ldcg(ws.klist + t), max_src, out);
@@ -1029,6 +1051,7 @@ __global__ void __launch_bounds__(G_THREADS) k_ccl_emit(CclWs ws, int32_t max_sr
 
 __global__ void __launch_bounds__(G_THREADS) k_tile_final(CclWs ws, int64_t W, int64_t H, int ntx, int32_t* labels) {
     __shared__ __align__(16) int32_t lab[T_TH * T_TW];
+    dep_begin();
     ccl_final_tile(ws, lab, blockIdx.x, W, H, ntx, labels);
 }
 
@@ -1259,6 +1282,7 @@ int ipp_launch_detect(const DetectArgs& A, cudaStream_t s) {
     J.mw = cdiv(A.W, 32);
     J.min_area = A.min_area;
     J.ws = w;
+    bool cleared = false;
     if (A.mode == MODE_MASK) {
         J.mask = A.mask_in;
     } else {  // subtract (fused) and threshold into the workspace's bit rows
@@ -1271,6 +1295,11 @@ int ipp_launch_detect(const DetectArgs& A, cudaStream_t s) {
         T.k = A.k; T.thresh_abs = A.thresh_abs; T.filter = false;
         T.mask = (uint32_t*)((unsigned char*)A.ws + L.off[24]);
         T.mw = J.mw;
+        // the kept-node counter, the overflow count and the per-tile-row counts start at
+        // zero: cleared by the threshold pass (the spline form and a given mask: below)
+        T.zero = A.interp == 1 ? nullptr : w.counters;
+        T.nzero = L.nty + CT_WORDS;
+        cleared = T.zero != nullptr;
         dim3 sg((unsigned)cdiv(A.W, ST_TW), (unsigned)cdiv(A.H, ST_TH));
         if (A.interp == 1) {
             if (A.filter) return ipp_set_error(IPP_ERR_NOT_SUPPORTED, "detection filter with the spline reading");
@@ -1278,54 +1307,56 @@ int ipp_launch_detect(const DetectArgs& A, cudaStream_t s) {
             dim3 spg((unsigned)cdiv(A.W, 128), (unsigned)cdiv(A.H, 8));
             k_sub_thresh_spline<<<spg, 256, 0, s>>>(T, A.bnodes, A.rnodes);
         } else if (A.mesh_w >= 16) {
-            k_sub_thresh_poly<<<sg, ST_THREADS, 0, s>>>(T);
+            ipp_launch_dep(k_sub_thresh_poly, sg, ST_THREADS, 0, s, T);
         } else {
-            k_sub_thresh<<<sg, ST_THREADS, 0, s>>>(T);
+            ipp_launch_dep(k_sub_thresh, sg, ST_THREADS, 0, s, T);
         }
         if (int e = ipp_check_launch("k_sub_thresh")) return e;
         if (A.filter) {  // detection filter: threshold again, on the smoothed sub just written
             SubThreshJob Tf = T;
             Tf.fused = false;
             Tf.filter = true;
-            k_sub_thresh<<<sg, ST_THREADS, 0, s>>>(Tf);
+            Tf.zero = nullptr;
+            ipp_launch_dep(k_sub_thresh, sg, ST_THREADS, 0, s, Tf);
             if (int e = ipp_check_launch("k_sub_thresh (filtered)")) return e;
         }
         J.mask = T.mask;
     }
-    cudaFuncSetAttribute(k_tile_label, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileFast));
-    cudaFuncSetAttribute(k_tile_label_full, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileFull));
+    if (int e = ipp_once_per_device(1, [] {
+            const cudaError_t e0 = cudaFuncSetAttribute(k_tile_label, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                        (int)sizeof(TileFast));
+            return e0 != cudaSuccess ? e0
+                                     : cudaFuncSetAttribute(k_tile_label_full,
+                                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                            (int)sizeof(TileFull));
+        }))
+        return e;
     dim3 tg(L.ntx, L.nty);
-    // the kept-node counter, the overflow count and the per-tile-row counts start at zero
-    if (cudaMemsetAsync(w.counters, 0, (size_t)(L.nty + CT_WORDS) * 4, s) != cudaSuccess) return ipp_check_launch("memset");
-    k_tile_label<<<tg, T_THREADS, sizeof(TileFast), s>>>(J);
+    if (!cleared && cudaMemsetAsync(w.counters, 0, (size_t)(L.nty + CT_WORDS) * 4, s) != cudaSuccess)
+        return ipp_check_launch("memset");
+    if (cleared) ipp_launch_dep(k_tile_label, tg, T_THREADS, sizeof(TileFast), s, J);
+    else k_tile_label<<<tg, T_THREADS, sizeof(TileFast), s>>>(J);   // after a memset: no kernel to depend on
     if (int e = ipp_check_launch("k_tile_label")) return e;
-    {
-        int dev0 = 0, nsm = 0;
-        cudaGetDevice(&dev0);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev0);
-        const int64_t fg = std::min<int64_t>(L.ntiles, (int64_t)std::max(nsm, 1) * 4);
-        k_tile_label_full<<<(unsigned)fg, T_THREADS, sizeof(TileFull), s>>>(J);
-        if (int e = ipp_check_launch("k_tile_label_full")) return e;
-    }
+    const int sms = ipp_sm_count();
+    ipp_launch_dep(k_tile_label_full, dim3((unsigned)std::min<int64_t>(L.ntiles, (int64_t)sms * 4)), T_THREADS,
+                   sizeof(TileFull), s, J);
+    if (int e = ipp_check_launch("k_tile_label_full")) return e;
     const unsigned nt = (unsigned)L.ntiles;
-    k_ccl_union<<<nt, G_THREADS, 0, s>>>(w, L.ntx, L.nty);
+    ipp_launch_dep(k_ccl_union, dim3(nt), G_THREADS, 0, s, w, L.ntx, L.nty);
     if (int e = ipp_check_launch("k_ccl_union")) return e;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const unsigned pg = (unsigned)std::max(sms, 1) * 4;  // grid-stride over the kept nodes
-    k_ccl_resolve<<<pg, G_THREADS, 0, s>>>(w);
+    const dim3 pg((unsigned)sms * 4);  // grid-stride over the kept nodes
+    ipp_launch_dep(k_ccl_resolve, pg, G_THREADS, 0, s, w);
     if (int e = ipp_check_launch("k_ccl_resolve")) return e;
-    k_ccl_count<<<nt, G_THREADS, 0, s>>>(w, A.W, L.ntx, A.min_area);
+    ipp_launch_dep(k_ccl_count, dim3(nt), G_THREADS, 0, s, w, A.W, L.ntx, A.min_area);
     if (int e = ipp_check_launch("k_ccl_count")) return e;
     const size_t lsm = (size_t)2 * T_TH * L.ntx * sizeof(int);
     if (lsm > 200 * 1024) return ipp_set_error(IPP_ERR_NOT_SUPPORTED, "frame too wide for the labeling pass");
-    cudaFuncSetAttribute(k_ccl_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
-    k_ccl_scan<<<L.nty, G_THREADS, lsm, s>>>(w, L.ntx, L.nty, A.n_src_dev);
+    if (lsm > 40 * 1024) cudaFuncSetAttribute(k_ccl_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm);
+    ipp_launch_dep(k_ccl_scan, dim3(L.nty), G_THREADS, lsm, s, w, L.ntx, L.nty, A.n_src_dev);
     if (int e = ipp_check_launch("k_ccl_scan")) return e;
-    k_ccl_emit<<<pg, G_THREADS, 0, s>>>(w, A.max_src, A.stats);
+    ipp_launch_dep(k_ccl_emit, pg, G_THREADS, 0, s, w, A.max_src, A.stats);
     if (int e = ipp_check_launch("k_ccl_emit")) return e;
-    k_tile_final<<<nt, G_THREADS, 0, s>>>(w, A.W, A.H, L.ntx, A.labels);
+    ipp_launch_dep(k_tile_final, dim3(nt), G_THREADS, 0, s, w, A.W, A.H, L.ntx, A.labels);
     return ipp_check_launch("k_tile_final");
 }
 

@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 #include <vector>
 
 #include "jobs.cuh"
@@ -25,6 +26,7 @@ constexpr int ANN_CAP = ANN_BOX * ANN_BOX;                 // 1225
 // NPL box pixels in registers and reloads them only when the anchor moves.
 template <int NPL>
 __global__ void __launch_bounds__(P_THREADS) k_centroid(CenJob J) {
+    dep_begin();
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * P_THREADS + threadIdx.x) >> 5;
     const int nw = (gridDim.x * P_THREADS) >> 5;
@@ -226,6 +228,7 @@ __device__ __forceinline__ void centroid_rows_body(const CenJob& J, int vb, int 
 
 template <int CB>
 __global__ void __launch_bounds__(P_THREADS) k_centroid_rows(CenJob J) {
+    dep_begin();
     centroid_rows_body<CB>(J, blockIdx.x, gridDim.x);
 }
 
@@ -684,7 +687,10 @@ __device__ __forceinline__ void aperture_body(const PhotJob& J, int vb, int nvb)
     }
 }
 
-__global__ void __launch_bounds__(P_THREADS) k_aperture(PhotJob J) { aperture_body(J, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(P_THREADS) k_aperture(PhotJob J) {
+    dep_begin();
+    aperture_body(J, blockIdx.x, gridDim.x);
+}
 
 // batched form: the same bodies over a table of frames
 template <int CB>
@@ -928,33 +934,40 @@ __global__ void __launch_bounds__(P_THREADS) k_auto_phot(AutoJob J) {
 
 using namespace ipp;
 
-static int persistent_blocks(cudaStream_t) {
-    int dev = 0, sms = 0;
+static int persistent_blocks(cudaStream_t) { return ipp_sm_count() * 4; }
+
+// A persistent grid of exactly the blocks that fit at once (one wave).  The query
+// costs the host about as much as a launch, so the last answer is kept for each
+// kernel and device (shared memory and blocks an SM in one word).
+template <class K>
+static int resident_blocks(K kernel, std::atomic<uint64_t> (&memo)[64], size_t smem) {
+    int dev = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms * 4 : 512;
+    const bool slot = dev >= 0 && dev < 64;
+    const uint64_t m = slot ? memo[dev].load(std::memory_order_relaxed) : 0;
+    int per = (int)(m & 0xffff);
+    if (per == 0 || (m >> 16) != smem) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, P_THREADS, smem) != cudaSuccess || per < 1) per = 1;
+        if (slot) memo[dev].store(((uint64_t)smem << 16) | (uint64_t)per, std::memory_order_relaxed);
+    }
+    return ipp_sm_count() * per;
 }
 
-// A persistent grid of exactly the blocks that fit at once (one wave).
-template <class K>
-static int resident_blocks(K kernel, size_t smem) {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, P_THREADS, smem) != cudaSuccess || per < 1) per = 1;
-    return (sms > 0 ? sms : 132) * per;
+// One call site per kernel: the memo belongs to the kernel (template argument).
+template <auto K, class Job>
+static void launch_resident(size_t smem, cudaStream_t s, const Job& job) {
+    static std::atomic<uint64_t> memo[64];
+    ipp_launch_dep(K, dim3((unsigned)resident_blocks(K, memo, smem)), P_THREADS, smem, s, job);
 }
 
 int ipp_launch_centroid(const CenJob& J, cudaStream_t s) {
     const int R = (int)floorf(J.rad + 0.5f);
     const int nbox = (2 * R + 1) * (2 * R + 1);
-    if (2 * R + 1 <= CR_SMALL)
-        k_centroid_rows<CR_SMALL><<<resident_blocks(k_centroid_rows<CR_SMALL>, 0), P_THREADS, 0, s>>>(J);
-    else if (2 * R + 1 <= CR_BOX)
-        k_centroid_rows<CR_BOX><<<resident_blocks(k_centroid_rows<CR_BOX>, 0), P_THREADS, 0, s>>>(J);
-    else if (nbox <= 32 * 4) k_centroid<4><<<resident_blocks(k_centroid<4>, 0), P_THREADS, 0, s>>>(J);
-    else if (nbox <= 32 * 8) k_centroid<8><<<resident_blocks(k_centroid<8>, 0), P_THREADS, 0, s>>>(J);
-    else k_centroid<0><<<persistent_blocks(s), P_THREADS, 0, s>>>(J);
+    if (2 * R + 1 <= CR_SMALL) launch_resident<k_centroid_rows<CR_SMALL>>(0, s, J);
+    else if (2 * R + 1 <= CR_BOX) launch_resident<k_centroid_rows<CR_BOX>>(0, s, J);
+    else if (nbox <= 32 * 4) launch_resident<k_centroid<4>>(0, s, J);
+    else if (nbox <= 32 * 8) launch_resident<k_centroid<8>>(0, s, J);
+    else ipp_launch_dep(k_centroid<0>, dim3((unsigned)persistent_blocks(s)), P_THREADS, 0, s, J);
     return ipp_check_launch("k_centroid");
 }
 
@@ -978,14 +991,16 @@ int ipp_launch_aperture(const PhotJob& J0, cudaStream_t s) {
     PhotJob J = J0;
     J.ann_cap = annulus_cap(J);
     const size_t dyn = (size_t)P_WARPS * J.ann_cap * sizeof(float);
-    cudaFuncSetAttribute(k_aperture, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-    k_aperture<<<resident_blocks(k_aperture, dyn), P_THREADS, dyn, s>>>(J);
+    // static and dynamic shared memory together: above 48 KB only with the attribute
+    if (dyn > 24 * 1024) cudaFuncSetAttribute(k_aperture, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
+    launch_resident<k_aperture>(dyn, s, J);
     return ipp_check_launch("k_aperture");
 }
 
 int ipp_launch_auto_phot(const AutoJob& J, cudaStream_t s) {
     if (J.max_src <= 0) return IPP_OK;
-    k_auto_phot<<<resident_blocks(k_auto_phot, 0), P_THREADS, 0, s>>>(J);
+    static std::atomic<uint64_t> memo[64];
+    k_auto_phot<<<resident_blocks(k_auto_phot, memo, 0), P_THREADS, 0, s>>>(J);
     return ipp_check_launch("k_auto_phot");
 }
 
