@@ -37,8 +37,9 @@ namespace ipp {
 // share a region, each holds its slice in shared memory (84 KB; two blocks an SM)
 // and a pass ends in one exchange over distributed shared memory: the counters or
 // extrema of all blocks are read by every block, which then take the same decision.
-// Bound by the passes' integer work per element.  100 regions of 168 K pixels:
-// 820 -> 460 us.  A region above NC slices is read from memory in every pass.
+// Bound by the passes' integer work per element, so a slice holds ordered 32-bit keys
+// and the passes work on 32 bits wherever that is exact.  100 regions of 168 K
+// pixels: 820 us with one block, 460 us in clusters on 64-bit keys, 328 us now.  A region above NC slices is read from memory in every pass.
 constexpr int SS_T = 512, SS_W = SS_T / 32, SS_NC = 8;
 constexpr int SS_SLICE = 21504;   // pixels of a slice: 84 KB beside 18 KB of counters, two blocks an SM
 
@@ -57,15 +58,20 @@ struct StampRegion {
     int64_t pitch, W, H;
     int x0, y0, rw, rh;   // the region [x0, x0 + rw) x [y0, y0 + rh)
     int t0, t1;           // this block's pixels of it (raster index)
-    bool cached;          // they are in shared memory
-    const float* cache;
+    bool cached;          // their keys are in shared memory
+    const uint32_t* cache;
     int buf;              // exchange buffer in turn
 };
 
-__device__ __forceinline__ float reg_r(const StampRegion& g, int t) {
-    if (g.cached) return g.cache[t - g.t0];
+// Key of a pixel: fkey of a finite value, STAMP_NONE (no finite value's key) otherwise
+constexpr uint32_t STAMP_NONE = 0xffffffffu;
+__device__ __forceinline__ uint32_t reg_load(const StampRegion& g, int t) {
     const int yy = t / g.rw;
-    return __ldg(g.R + (int64_t)(g.y0 + yy) * g.pitch + (g.x0 + (t - yy * g.rw)));
+    const float v = __ldg(g.R + (int64_t)(g.y0 + yy) * g.pitch + (g.x0 + (t - yy * g.rw)));
+    return isfinite(v) ? fkey(v) : STAMP_NONE;
+}
+__device__ __forceinline__ uint32_t reg_key(const StampRegion& g, int t) {
+    return g.cached ? g.cache[t - g.t0] : reg_load(g, t);
 }
 
 // One exchange: this block's value(s) in S.xch[buf] are combined over the
@@ -105,47 +111,66 @@ __device__ __forceinline__ unsigned long long stamp_all(StampShared& S, int buf,
     return v;
 }
 
-// Keys of a region's finite values for the order statistics, as unsigned
-// 64-bit integers ordered like the quantities they stand for:
-//   mode 0: the value, fkey(v);
-//   mode 1: |v - med| exactly, as the integer |v 2^-e0 - med 2^-e0| -- every value
-//     and med are multiples of 2^e0 (e0: one below the smallest ulp in the
-//     region), so the difference is exact and its FP64 rounding is the FP64
-//     subtraction's, without FP64 arithmetic per element; the scaling is two exact
-//     products with powers of two, 2^-e0 = s1 s2 (shifting the significand instead
-//     of converting the product measured slower, 480 against 460 us);
-//   mode 2: the bit pattern of the FP64 |v - med| (when the region's range does
-//     not fit 62 bits at scale 2^e0).
-struct KeySpec {
-    int mode;
-    int e0;
-    float s1, s2;
-    double med;
-    long long imed;
-};
-
-__device__ __forceinline__ bool stamp_key(const StampRegion& g, int t, const KeySpec& ks, unsigned long long* k) {
-    const float v = reg_r(g, t);
-    if (!isfinite(v)) return false;
-    if (ks.mode == 0) {
-        *k = fkey(v);
-    } else if (ks.mode == 1) {
-        const long long d = __float2ll_rz(__fmul_rn(__fmul_rn(v, ks.s1), ks.s2)) - ks.imed;
-        *k = (unsigned long long)(d < 0 ? -d : d);
-    } else {
-        *k = (unsigned long long)__double_as_longlong(fabs((double)v - ks.med));
+// Keys of a region's finite values for the order statistics, as unsigned integers
+// ordered like the quantities they stand for:
+//   value, 32 bits: fkey(v);
+//   |v - med| exactly, as the integer |v 2^-e0 - med 2^-e0| -- every value and med are
+//     multiples of 2^e0 (e0: one below the smallest ulp in the region), so the
+//     difference is exact and its FP64 rounding is the FP64 subtraction's, without
+//     FP64 arithmetic per element; the scaling is two exact products with powers of
+//     two, 2^-e0 = s1 s2;
+//   the same in 32 bits: the conversion saturates at +-2^31, so a key below
+//     2^31 - 1 - |med 2^-e0| is exact and every other pixel's is at least that.  Few
+//     pixels of a region are far from its median: the MAD's keys nearly always are
+//     below, and these passes take half the instructions of the 64-bit ones;
+//   the bit pattern of the FP64 |v - med| (when the region's range does not fit 62
+//     bits at scale 2^e0).
+struct ValueKey {
+    using T = uint32_t;
+    __device__ __forceinline__ bool operator()(uint32_t k, T* out) const {
+        *out = k;
+        return k != STAMP_NONE;
     }
-    return true;
-}
+};
+struct DistKey32 {
+    using T = uint32_t;
+    float s1, s2;
+    int imed;
+    __device__ __forceinline__ bool operator()(uint32_t k, T* out) const {
+        const int v = __float2int_rz(__fmul_rn(__fmul_rn(fkey_inv(k), s1), s2));
+        *out = v < imed ? (uint32_t)imed - (uint32_t)v : (uint32_t)v - (uint32_t)imed;
+        return k != STAMP_NONE;
+    }
+};
+struct DistKey64 {
+    using T = unsigned long long;
+    float s1, s2;
+    long long imed;
+    __device__ __forceinline__ bool operator()(uint32_t k, T* out) const {
+        const long long d = __float2ll_rz(__fmul_rn(__fmul_rn(fkey_inv(k), s1), s2)) - imed;
+        *out = (T)(d < 0 ? -d : d);
+        return k != STAMP_NONE;
+    }
+};
+struct DistKeyD {
+    using T = unsigned long long;
+    double med;
+    __device__ __forceinline__ bool operator()(uint32_t k, T* out) const {
+        *out = (T)__double_as_longlong(fabs((double)fkey_inv(k) - med));
+        return k != STAMP_NONE;
+    }
+};
 
 // The k-th smallest key (0-based) of the region: radix selection, 8 bits a
 // pass from bit top + 7 down, every key sharing the bits above top with
 // prefix0; per-warp histograms in shared memory, fed by per-thread run lengths
 // of equal digits, summed over the block, then over the cluster.
-__device__ unsigned long long region_select(StampRegion& g, const KeySpec& ks, long long k, int top,
+template <class Key>
+__device__ unsigned long long region_select(StampRegion& g, const Key& key_of, long long k, int top,
                                             unsigned long long prefix0, StampShared& S) {
+    using T = typename Key::T;
     auto cl = cooperative_groups::this_cluster();
-    unsigned long long prefix = prefix0;
+    T prefix = (T)prefix0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int shift = top; shift >= 0; shift -= 8) {
         for (int t = threadIdx.x; t < SS_W * 256; t += SS_T) S.hist[t] = 0;
@@ -154,11 +179,11 @@ __device__ unsigned long long region_select(StampRegion& g, const KeySpec& ks, l
         // keys mostly share their high digits) and adds a run to its warp's
         // histogram when the digit changes
         unsigned cur = 256u, run = 0u;
+        const bool all = shift + 8 >= 8 * (int)sizeof(T);   // the first digit: no bits above it
         for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
-            unsigned long long key = 0;
-            bool ok = stamp_key(g, t, ks, &key);
-            if (ok && shift + 8 < 64) ok = (key >> (shift + 8)) == prefix;
-            if (!ok) continue;
+            T key;
+            const bool ok = key_of(reg_key(g, t), &key);
+            if (!ok || !(all || (key >> (shift + 8)) == prefix)) continue;
             const unsigned dig = (unsigned)((key >> shift) & 255u);
             if (dig == cur) {
                 run++;
@@ -207,7 +232,7 @@ __device__ unsigned long long region_select(StampRegion& g, const KeySpec& ks, l
             }
         }
         __syncthreads();
-        prefix = (prefix << 8) | (unsigned long long)S.sdig;
+        prefix = (T)(prefix << 8) | (T)S.sdig;
         k -= S.sbelow;
         __syncthreads();
     }
@@ -217,22 +242,27 @@ __device__ unsigned long long region_select(StampRegion& g, const KeySpec& ks, l
 // the two middle order statistics (k0 = (n - 1) / 2, k1 = n / 2) as keys, for
 // keys in [kmin, kmax]: the radix passes start at the highest byte where kmin
 // and kmax differ
-__device__ void region_middle(StampRegion& g, const KeySpec& ks, long long n, unsigned long long kmin,
+template <class Key>
+__device__ void region_middle(StampRegion& g, const Key& key_of, long long n, unsigned long long kmin,
                               unsigned long long kmax, StampShared& S, unsigned long long* a, unsigned long long* b) {
+    using T = typename Key::T;
     const long long k0 = (n - 1) / 2, k1 = n / 2;
     const unsigned long long dif = kmin ^ kmax;
     const int top = dif ? ((63 - __clzll((long long)dif)) & ~7) : 0;
     const unsigned long long prefix0 = top + 8 < 64 ? kmin >> (top + 8) : 0ull;
-    *a = region_select(g, ks, k0, top, prefix0, S);
+    *a = region_select(g, key_of, k0, top, prefix0, S);
     if (k1 == k0) { *b = *a; return; }
     // count of keys <= a, smallest key > a
-    unsigned long long c = 0, nx = ~0ull;
+    uint32_t cnt = 0;
+    T next = (T)~(T)0;
+    const T ka = (T)*a;
     for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
-        unsigned long long key;
-        if (!stamp_key(g, t, ks, &key)) continue;
-        if (key <= *a) c++;
-        else if (key < nx) nx = key;
+        T key;
+        if (!key_of(reg_key(g, t), &key)) continue;
+        if (key <= ka) cnt++;
+        else if (key < next) next = key;
     }
+    unsigned long long c = cnt, nx = next;
     stamp_part(S, 0, c, OpAdd());
     stamp_part(S, 1, nx, OpMin());
     __syncthreads();
@@ -261,7 +291,7 @@ __device__ bool block_box_finite(const float* A, int64_t pitch, int x, int y, in
 __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const float* R, int64_t W, int64_t H,
                                                         int64_t pitch, int nsx, int nsy, int hw, int fh, double nsig,
                                                         int slice, int2* reg_out) {
-    extern __shared__ float stamp_cache[];   // [slice]
+    extern __shared__ uint32_t stamp_cache[];   // [slice]
     __shared__ StampShared S;
     auto cl = cooperative_groups::this_cluster();
     const int nc = (int)cl.num_blocks(), rank = (int)cl.block_rank();
@@ -283,14 +313,13 @@ __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const fl
     // the finite values: count, key range, smallest ulp exponent, largest |v|
     uint32_t c = 0, kmin = ~0u, kmax = 0, emin = ~0u, amax = 0;
     for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
-        const float v = reg_r(g, t);
-        if (fits) stamp_cache[t - g.t0] = v;
-        if (!isfinite(v)) continue;
+        const uint32_t k = reg_load(g, t);
+        if (fits) stamp_cache[t - g.t0] = k;
+        if (k == STAMP_NONE) continue;
         c++;
-        const uint32_t k = fkey(v);
         kmin = min(kmin, k);
         kmax = max(kmax, k);
-        const uint32_t bits = __float_as_uint(v) & 0x7fffffffu;
+        const uint32_t bits = __float_as_uint(fkey_inv(k)) & 0x7fffffffu;
         emin = min(emin, max(bits >> 23, 1u));      // ulp 2^(be - 150), denormals as be = 1
         amax = max(amax, bits);
     }
@@ -318,33 +347,36 @@ __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const fl
         return;
     }
     // median (Eq. 1's even-count mean of the middle pair)
-    KeySpec ks{0, 0, 1.f, 1.f, 0.0, 0};
     unsigned long long ka, kb;
-    region_middle(g, ks, n, gmin, gmax, S, &ka, &kb);
+    region_middle(g, ValueKey{}, n, gmin, gmax, S, &ka, &kb);
     const double va = (double)fkey_inv((uint32_t)ka), vb = (double)fkey_inv((uint32_t)kb);
     const double med = (n & 1) ? vb : __dmul_rn(0.5, __dadd_rn(va, vb));
     // MAD: exact integer differences at scale 2^e0 when they fit 62 bits
-    ks.med = med;
-    ks.e0 = (int)emin - 150 - 1;
-    const double span = ldexp((double)__uint_as_float(amax) + fabs(med), -ks.e0);
-    double mad;
+    const int e0 = (int)emin - 150 - 1;
+    const double span = ldexp((double)__uint_as_float(amax) + fabs(med), -e0);
+    double da, db;
     if (span < 4.6e18) {
-        ks.mode = 1;
         // -150 <= e0 <= 103: two powers of two within the normal range, of one sign
-        const int h1 = -ks.e0 / 2, h2 = -ks.e0 - h1;
-        ks.s1 = __uint_as_float((uint32_t)(h1 + 127) << 23);
-        ks.s2 = __uint_as_float((uint32_t)(h2 + 127) << 23);
-        ks.imed = __double2ll_rz(ldexp(med, -ks.e0));
+        const int h1 = -e0 / 2, h2 = -e0 - h1;
+        const float s1 = __uint_as_float((uint32_t)(h1 + 127) << 23), s2 = __uint_as_float((uint32_t)(h2 + 127) << 23);
+        const long long imed = __double2ll_rz(ldexp(med, -e0));
         const unsigned long long top = (unsigned long long)span + 1ull;
-        region_middle(g, ks, n, 0ull, top, S, &ka, &kb);
-        const double da = ldexp((double)ka, ks.e0), db = ldexp((double)kb, ks.e0);
-        mad = (n & 1) ? db : __dmul_rn(0.5, __dadd_rn(da, db));
+        // the same in every block: n, med, the extrema and the selected keys are the region's
+        const long long exact32 = 2147483647ll - (imed < 0 ? -imed : imed);
+        bool done = false;
+        if (exact32 > 0) {
+            region_middle(g, DistKey32{s1, s2, (int)imed}, n, 0ull, top < 0xffffffffull ? top : 0xffffffffull, S, &ka, &kb);
+            done = (long long)kb < exact32;
+        }
+        if (!done) region_middle(g, DistKey64{s1, s2, imed}, n, 0ull, top, S, &ka, &kb);
+        da = ldexp((double)ka, e0);
+        db = ldexp((double)kb, e0);
     } else {
-        ks.mode = 2;
-        region_middle(g, ks, n, 0ull, ~0ull, S, &ka, &kb);
-        const double da = __longlong_as_double((long long)ka), db = __longlong_as_double((long long)kb);
-        mad = (n & 1) ? db : __dmul_rn(0.5, __dadd_rn(da, db));
+        region_middle(g, DistKeyD{med}, n, 0ull, ~0ull, S, &ka, &kb);
+        da = __longlong_as_double((long long)ka);
+        db = __longlong_as_double((long long)kb);
     }
+    const double mad = (n & 1) ? db : __dmul_rn(0.5, __dadd_rn(da, db));
     const double sgm = __dmul_rn(1.4826, mad);
     const double thr = __dadd_rn(med, __dmul_rn(nsig, sgm));
     // the brightest eligible pixel: arg-max rounds over the keys below the last
@@ -356,10 +388,8 @@ __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const fl
     for (;;) {
         unsigned long long mk = 0;
         for (int t = g.t0 + threadIdx.x; t < g.t1; t += SS_T) {
-            const float v = reg_r(g, t);
-            if (!isfinite(v)) continue;
-            const uint32_t fk = fkey(v);
-            if (fk < (uint32_t)(mk >> 32) || fk > (uint32_t)(bound >> 32)) continue;
+            const uint32_t fk = reg_key(g, t);
+            if (fk == STAMP_NONE || fk < (uint32_t)(mk >> 32) || fk > (uint32_t)(bound >> 32)) continue;
             const int yy = t / g.rw, y = g.y0 + yy, x = g.x0 + (t - yy * g.rw);
             if (x < m || y < m || x > W - 1 - m || y > H - 1 - m) continue;
             const unsigned long long key =
