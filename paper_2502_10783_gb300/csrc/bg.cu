@@ -118,7 +118,7 @@ __device__ __forceinline__ bool mesh_value_at(const GG& G, int r, int c, float* 
 // re-reads see identical values.
 // The quads of a raw frame: 8 bytes of the frame and 16 of the inverse flat (and of
 // the bias map) a load, where the scalar path takes four loads of each and their
-// addresses.  4096 x 4096 raw frame, 128 px meshes: k_mesh_stats 206 -> @MS16@ us.
+// addresses.  4096 x 4096 raw frame, 128 px meshes: k_mesh_stats 206 -> 120 us.
 template <int T, class F>
 __device__ __forceinline__ void mesh_for_each_u16(const MeshGeom& G, F& f) {
     constexpr int VCH = 2;
