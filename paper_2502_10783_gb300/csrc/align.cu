@@ -86,6 +86,7 @@ __device__ __forceinline__ double sip_val(const double* c, int order, double u, 
 // polynomials and nine divisions a node and Newton step, before).
 __global__ void __launch_bounds__(AL_T) k_wcs_map(WcsPair P, int64_t nx, int64_t ny, int step,
                                                   double* __restrict__ xo, double* __restrict__ yo) {
+    dep_begin();
     const WcsDev &src = P.src, &tgt = P.tgt;
     const double* R = P.R;
     const int64_t n = nx * ny;
@@ -189,6 +190,7 @@ __device__ __forceinline__ unsigned int* aff_done(double* part1) { return reinte
 // pass 1: per-block count and coordinate sums
 template <int T>
 __global__ void __launch_bounds__(T) k_aff_sum1(AffPts P, double* __restrict__ part) {
+    dep_begin();
     __shared__ double red[5][T / 32];
     double v[5] = {0, 0, 0, 0, 0};
     if (blockIdx.x == 0 && threadIdx.x == 0) *aff_done(part) = 0u;
@@ -245,6 +247,7 @@ __device__ void aff_solve(const double s[5], double saa, double sa, double sb, d
 template <int T>
 __global__ void __launch_bounds__(T) k_aff_sum2(AffPts P, double* __restrict__ part1, double* __restrict__ part2,
                                                    double* __restrict__ M, int32_t* __restrict__ status) {
+    dep_begin();
     __shared__ double red[3][T / 32];
     __shared__ double cs[5], mean[4], mom[3];
     __shared__ bool last;
@@ -345,6 +348,7 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ sr
                                                     int64_t pitch, const double* __restrict__ Minv, int64_t Wo,
                                                     int64_t Ho, float fill, float* __restrict__ out,
                                                     int64_t opitch, bool vout) {
+    dep_begin();
     // the transform as double-floats, converted once per block: FP64 work on
     // this GPU's narrow FP64 pipe stays off the per-pixel and per-segment path
     __shared__ float mh[6], ml[6];
@@ -500,7 +504,7 @@ int ipp_launch_wcs_map(const ipp_wcs& src, const ipp_wcs& tgt, int64_t nx, int64
     P.icd[2] = -tgt.cd[2] * k;
     P.icd[3] = tgt.cd[0] * k;
     // FP64-bound: 64-thread blocks so that small node grids still reach every SM
-    k_wcs_map<<<al_grid(64, nx * ny, 16), 64, 0, s>>>(P, nx, ny, step, xo, yo);
+    ipp_launch_dep(k_wcs_map, dim3(al_grid(64, nx * ny, 16)), 64, 0, s, P, nx, ny, step, xo, yo);
     return ipp_check_launch("k_wcs_map");
 }
 
@@ -514,13 +518,13 @@ int ipp_launch_affine_fit(const double* x, const double* y, const double* xt, co
     // two warps a block while a thread has at most eight points; beyond that the
     // loads of eight warps are wanted in flight
     if (n <= (int64_t)8 * AF_BLOCKS * AF_SMALL) {
-        k_aff_sum1<AF_SMALL><<<AF_BLOCKS, AF_SMALL, 0, s>>>(P, p1);
+        ipp_launch_dep(k_aff_sum1<AF_SMALL>, dim3(AF_BLOCKS), AF_SMALL, 0, s, P, p1);
         if (int e = ipp_check_launch("k_aff_sum1")) return e;
-        k_aff_sum2<AF_SMALL><<<AF_BLOCKS, AF_SMALL, 0, s>>>(P, p1, p2, M, status);
+        ipp_launch_dep(k_aff_sum2<AF_SMALL>, dim3(AF_BLOCKS), AF_SMALL, 0, s, P, p1, p2, M, status);
     } else {
-        k_aff_sum1<AF_LARGE><<<AF_BLOCKS, AF_LARGE, 0, s>>>(P, p1);
+        ipp_launch_dep(k_aff_sum1<AF_LARGE>, dim3(AF_BLOCKS), AF_LARGE, 0, s, P, p1);
         if (int e = ipp_check_launch("k_aff_sum1")) return e;
-        k_aff_sum2<AF_LARGE><<<AF_BLOCKS, AF_LARGE, 0, s>>>(P, p1, p2, M, status);
+        ipp_launch_dep(k_aff_sum2<AF_LARGE>, dim3(AF_BLOCKS), AF_LARGE, 0, s, P, p1, p2, M, status);
     }
     return ipp_check_launch("k_aff_sum2");
 }
@@ -529,7 +533,7 @@ int ipp_launch_reproject(const float* src, int64_t W, int64_t H, int64_t pitch, 
                          int64_t Ho, float fill, float* out, int64_t opitch, cudaStream_t s) {
     const bool vout = (opitch % 4 == 0) && (((uintptr_t)out & 15) == 0);
     const int64_t tasks = ((Wo + RP_SEG - 1) / RP_SEG) * Ho;
-    k_reproject<<<al_grid(AL_T / 32 * RP_GRP, tasks, 8), AL_T, 0, s>>>(src, W, H, pitch, Minv, Wo, Ho, fill, out, opitch,
+    ipp_launch_dep(k_reproject, dim3(al_grid(AL_T / 32 * RP_GRP, tasks, 8)), AL_T, 0, s, src, W, H, pitch, Minv, Wo, Ho, fill, out, opitch,
                                                                         vout);
     return ipp_check_launch("k_reproject");
 }

@@ -680,7 +680,7 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
 #pragma unroll
         for (int j = 0; j < 8; j++) {
             const int k = lane + 32 * j;
-            const int r = (int)(((int64_t)k * G.he) >> 8), c = (int)(((int64_t)k * 61 + 7) % G.we);
+            const int r = (k * G.he) >> 8, c = (k * 61 + 7) % G.we;   // he <= 16384
             float x;
             a[j] = mesh_value_at(G, r, c, &x) ? x : INFINITY;
             nv += a[j] != INFINITY;
@@ -735,7 +735,12 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
         if (lane == 0) { S.redf[warp] = vmin; S.redf[MS_WARPS + warp] = vmax; }
     }
     __syncthreads();
-    float mu0 = 0.f, sd0 = 0.f;  // mean and sigma of the mesh (warp 0; used only to re-place a missed window)
+    // sums of read 1 (lane 0 of warp 0): their mean and sigma re-place a missed window,
+    // and only then pay for FP64 arithmetic on the serial path (10 K cycles a mesh)
+    long long r1_i1 = 0, r1_i2 = 0;
+    df r1_o1{0.f, 0.f}, r1_o2{0.f, 0.f};
+    const int e_r1 = e;
+    const float c_r1 = cstar;
     if (warp == 0) {
         int c[3];
         long long i1, i2;
@@ -747,13 +752,7 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
             S.bc_i[BI_N0] = c[0];
             S.bc_f[2] = a;
             S.bc_f[3] = b;
-            if (c[0] > 0) {
-                const double unit0 = ldexp(1.0, e - MS_SCALE_BITS);
-                const double m1 = ((double)i1 * unit0 + df_to_d(o1)) / c[0];
-                const double var = ((double)i2 * unit0 * unit0 + df_to_d(o2)) / c[0] - m1 * m1;
-                mu0 = (float)((double)cstar + m1);
-                sd0 = (float)sqrt(fmax(var, 0.0));
-            }
+            r1_i1 = i1; r1_i2 = i2; r1_o1 = o1; r1_o2 = o2;
         }
     }
     __syncthreads();
@@ -796,6 +795,10 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
                 const int b16 = bq[0], b50 = bq[1], b84 = bq[2];
                 const int ends = (int)(S.hbuf[0] + S.hbuf[MS_NB + 1]);
                 if (round < 2 && ((round == 0 && S.bc_i[BI_SBAD]) || b50 == 0 || b50 == MS_NB + 1 || ends > n0 / 8)) {
+                    const double unit0 = ldexp(1.0, e_r1 - MS_SCALE_BITS);
+                    const double m1 = ((double)r1_i1 * unit0 + df_to_d(r1_o1)) / n0;
+                    const double var = ((double)r1_i2 * unit0 * unit0 + df_to_d(r1_o2)) / n0 - m1 * m1;
+                    const float mu0 = (float)((double)c_r1 + m1), sd0 = (float)sqrt(fmax(var, 0.0));
                     float span = fmaxf(8.0f * sd0, (vmax - vmin) * 1e-6f);
                     span = fmaxf(span, fabsf(mu0) * 1e-6f + 1e-30f);
                     const int e2 = max(min((int)floorf(log2f(span / MS_NB)), 100), -110);

@@ -102,6 +102,7 @@ __device__ __forceinline__ df pair32_value(const long long* p) {
 
 // barycentres (exact sums, double-float quotient)
 __global__ void __launch_bounds__(CL_T) k_clean_obj_a(const int32_t* n_dev, int32_t max_obj, CleanWs ws) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int l = blockIdx.x * CL_T + threadIdx.x; l <= n; l += gridDim.x * CL_T) {
         if (l == 0) continue;
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_obj_a(const int32_t* n_dev, int3
 __global__ void __launch_bounds__(CL_T) k_clean_pix_b(const float* sub, int64_t pitch, const int32_t* labels,
                                                       int64_t W, int64_t H, const int32_t* n_dev, int32_t max_obj,
                                                       CleanWs ws) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int64_t p = (int64_t)blockIdx.x * CL_T + threadIdx.x; p < W * H; p += (int64_t)gridDim.x * CL_T) {
         const int l = __ldg(labels + p);
@@ -173,6 +175,7 @@ __device__ float clean_thr_at(const CleanThr& T, int64_t x, int64_t y) {
 // moments, the model's inverse shape, and the threshold at the peak pixel
 __global__ void __launch_bounds__(CL_T) k_clean_obj_b(const int32_t* n_dev, int32_t max_obj, CleanWs ws,
                                                       CleanThr T, float inv_a2) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int l = blockIdx.x * CL_T + threadIdx.x; l <= n; l += gridDim.x * CL_T) {
         if (l == 0) continue;
@@ -206,6 +209,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_obj_b(const int32_t* n_dev, int3
 constexpr int BS_T = 1024, BS_N = 2 * BS_T;
 
 __global__ void __launch_bounds__(CL_T) k_clean_keys(const int32_t* n_dev, int32_t max_obj, CleanWs ws, int P) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int r = blockIdx.x * CL_T + threadIdx.x; r < P; r += gridDim.x * CL_T) {
         const int l = r + 1;
@@ -223,6 +227,7 @@ __device__ __forceinline__ void bitonic_cas(unsigned long long& a, unsigned long
 // k in [k_lo, k_hi] (powers of two), strides below BS_N only; k_lo = 2 sorts the
 // block from scratch, k_lo = k_hi finishes one merge of size k
 __global__ void __launch_bounds__(BS_T) k_bitonic_local(unsigned long long* keys, int k_lo, int k_hi) {
+    dep_begin();
     __shared__ unsigned long long sk[BS_N];
     const int base = blockIdx.x * BS_N;
     sk[threadIdx.x] = keys[base + threadIdx.x];
@@ -242,6 +247,7 @@ __global__ void __launch_bounds__(BS_T) k_bitonic_local(unsigned long long* keys
 }
 
 __global__ void __launch_bounds__(CL_T) k_bitonic_global(unsigned long long* keys, int P, int k, int j) {
+    dep_begin();
     const int t = blockIdx.x * CL_T + threadIdx.x;
     if (t >= P / 2) return;
     const int i = 2 * t - (t & (j - 1));
@@ -277,9 +283,18 @@ __device__ __forceinline__ void kahan_acc(float& s, float& c, float v) {
     s = t;
 }
 
+// a / b by the hardware's reciprocal without the steps that extend it to subnormals
+// (a pair's profile is never near 2^-126)
+__device__ __forceinline__ float div_ftz(float a, float b) {
+    float y;
+    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+
 template <bool UNIT>
 __global__ void __launch_bounds__(CL_T) k_clean_pairs(const int32_t* n_dev, int32_t max_obj, CleanWs ws, int64_t W,
                                                       float beta) {
+    dep_begin();
     __shared__ float4 sa[CL_T], sq[CL_T];   // (cx, cy, peak, lo.x), (y2', -2 xy', x2', lo.y) of object rank t
     __shared__ int sb[CL_T];                // its label
     const int n = clean_n(n_dev, max_obj);
@@ -316,12 +331,13 @@ __global__ void __launch_bounds__(CL_T) k_clean_pairs(const int32_t* n_dev, int3
         }
         __syncthreads();
         const int m = min(CL_T, lim - t0);
+#pragma unroll 4
         for (int t = 0; t < m; t++) {
             const float4 a = sa[t], e = sq[t];
             const float dx = (px - a.x) - a.w, dy = (py - a.y) - e.w;
             // r^2 / a^2 = dx (y2' dx - 2 xy' dy) + x2' dy^2
             const float q = fmaf(dx, fmaf(e.x, dx, e.y * dy), e.z * dy * dy);
-            const float mv = UNIT ? __fdividef(a.z, 1.0f + q) : a.z * expf(-beta * log1pf(q));
+            const float mv = UNIT ? div_ftz(a.z, 1.0f + q) : a.z * expf(-beta * log1pf(q));
             kahan_acc(sum, comp, mv);
             if (mv >= best) {                              // ties to the smaller label (rare)
                 const int lj = sb[t];
@@ -334,6 +350,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_pairs(const int32_t* n_dev, int3
 
 // per rank: the chunks' partials in chunk order, the decision and the target
 __global__ void __launch_bounds__(CL_T) k_clean_decide(const int32_t* n_dev, int32_t max_obj, CleanWs ws) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int r = blockIdx.x * CL_T + threadIdx.x; r < n; r += gridDim.x * CL_T) {
         const unsigned long long key = ws.skey[r];
@@ -354,6 +371,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_decide(const int32_t* n_dev, int
 }
 
 __global__ void __launch_bounds__(CL_T) k_clean_into_init(const int32_t* n_dev, int32_t max_obj, CleanWs ws) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int l = blockIdx.x * CL_T + threadIdx.x; l <= n; l += gridDim.x * CL_T) ws.into[l] = l;
 }
@@ -361,6 +379,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_into_init(const int32_t* n_dev, 
 // merge targets followed to a kept object (each target is strictly brighter, so
 // a chain has at most n steps): num[i] = that object
 __global__ void __launch_bounds__(CL_T) k_clean_root(const int32_t* n_dev, int32_t max_obj, CleanWs ws) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int i = blockIdx.x * CL_T + threadIdx.x + 1; i <= n; i += gridDim.x * CL_T) {
         int r = i;
@@ -371,6 +390,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_root(const int32_t* n_dev, int32
 
 // kept objects (their own root, holding pixels) per tile of 1024 labels
 __global__ void __launch_bounds__(1024) k_clean_count(const int32_t* n_dev, int32_t max_obj, CleanWs ws) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     const int i = blockIdx.x * 1024 + threadIdx.x + 1;
     const int kept = (i <= n && ws.num[i] == i && ws.geo[i].w > 0.f) ? 1 : 0;
@@ -383,6 +403,7 @@ __global__ void __launch_bounds__(1024) k_clean_count(const int32_t* n_dev, int3
 // (self) target in into[]; the count goes to n_out.
 __global__ void __launch_bounds__(1024) k_clean_assign(const int32_t* n_dev, int32_t max_obj, CleanWs ws,
                                                        int32_t* n_out) {
+    dep_begin();
     __shared__ int red[32];
     const int n = clean_n(n_dev, max_obj);
     const int tile = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -413,6 +434,7 @@ __global__ void __launch_bounds__(1024) k_clean_assign(const int32_t* n_dev, int
 
 __global__ void __launch_bounds__(CL_T) k_clean_relabel(const int32_t* labels, int64_t npx, const int32_t* n_dev,
                                                         int32_t max_obj, CleanWs ws, int32_t* out) {
+    dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int64_t p = (int64_t)blockIdx.x * CL_T + threadIdx.x; p < npx; p += (int64_t)gridDim.x * CL_T) {
         const int l = __ldg(labels + p);
@@ -482,44 +504,44 @@ int ipp_launch_clean(const float* sub, int64_t pitch, const int32_t* labels, int
     const float a2 = (float)(2.0 * std::log(2.0) / (std::pow(2.0, 1.0 / beta) - 1.0));
     k_clean_pix_a<<<pg, CL_T, 0, s>>>(sub, pitch, labels, W, H, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_pix_a")) return e;
-    k_clean_obj_a<<<og, CL_T, 0, s>>>(n_dev, max_obj, w);
+    ipp_launch_dep(k_clean_obj_a, dim3(og), CL_T, 0, s, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_obj_a")) return e;
-    k_clean_pix_b<<<pg, CL_T, 0, s>>>(sub, pitch, labels, W, H, n_dev, max_obj, w);
+    ipp_launch_dep(k_clean_pix_b, dim3(pg), CL_T, 0, s, sub, pitch, labels, W, H, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_pix_b")) return e;
     const CleanThr T{thr_map, mesh_rms, nx, ny, mesh_w, mesh_h, k, thresh_abs, W};
-    k_clean_obj_b<<<og, CL_T, 0, s>>>(n_dev, max_obj, w, T, 1.0f / a2);
+    ipp_launch_dep(k_clean_obj_b, dim3(og), CL_T, 0, s, n_dev, max_obj, w, T, 1.0f / a2);
     if (int e = ipp_check_launch("k_clean_obj_b")) return e;
-    k_clean_into_init<<<og, CL_T, 0, s>>>(n_dev, max_obj, w);
+    ipp_launch_dep(k_clean_into_init, dim3(og), CL_T, 0, s, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_into_init")) return e;
     // brightness order: keys, 2048-key blocks sorted in shared memory, then the
     // merges of 4096 keys and more
     const int P = w.P;
-    k_clean_keys<<<(unsigned)(P / CL_T), CL_T, 0, s>>>(n_dev, max_obj, w, P);
+    ipp_launch_dep(k_clean_keys, dim3((unsigned)(P / CL_T)), CL_T, 0, s, n_dev, max_obj, w, P);
     if (int e = ipp_check_launch("k_clean_keys")) return e;
-    k_bitonic_local<<<(unsigned)(P / BS_N), BS_T, 0, s>>>(w.skey, 2, BS_N);
+    ipp_launch_dep(k_bitonic_local, dim3((unsigned)(P / BS_N)), BS_T, 0, s, w.skey, 2, BS_N);
     if (int e = ipp_check_launch("k_bitonic_local")) return e;
     for (int kk = 2 * BS_N; kk <= P; kk <<= 1) {
         for (int j = kk >> 1; j >= BS_N; j >>= 1) {
-            k_bitonic_global<<<(unsigned)(P / 2 / CL_T), CL_T, 0, s>>>(w.skey, P, kk, j);
+            ipp_launch_dep(k_bitonic_global, dim3((unsigned)(P / 2 / CL_T)), CL_T, 0, s, w.skey, P, kk, j);
             if (int e = ipp_check_launch("k_bitonic_global")) return e;
         }
-        k_bitonic_local<<<(unsigned)(P / BS_N), BS_T, 0, s>>>(w.skey, kk, kk);
+        ipp_launch_dep(k_bitonic_local, dim3((unsigned)(P / BS_N)), BS_T, 0, s, w.skey, kk, kk);
         if (int e = ipp_check_launch("k_bitonic_local")) return e;
     }
     const int nchunk = (P + CL_JC - 1) / CL_JC;
     const dim3 pg2((unsigned)(P / CL_T), (unsigned)nchunk);
-    if (beta == 1.0f) k_clean_pairs<true><<<pg2, CL_T, 0, s>>>(n_dev, max_obj, w, W, beta);
-    else k_clean_pairs<false><<<pg2, CL_T, 0, s>>>(n_dev, max_obj, w, W, beta);
+    if (beta == 1.0f) ipp_launch_dep(k_clean_pairs<true>, dim3(pg2), CL_T, 0, s, n_dev, max_obj, w, W, beta);
+    else ipp_launch_dep(k_clean_pairs<false>, dim3(pg2), CL_T, 0, s, n_dev, max_obj, w, W, beta);
     if (int e = ipp_check_launch("k_clean_pairs")) return e;
-    k_clean_decide<<<og, CL_T, 0, s>>>(n_dev, max_obj, w);
+    ipp_launch_dep(k_clean_decide, dim3(og), CL_T, 0, s, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_decide")) return e;
-    k_clean_root<<<og, CL_T, 0, s>>>(n_dev, max_obj, w);
+    ipp_launch_dep(k_clean_root, dim3(og), CL_T, 0, s, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_root")) return e;
     const unsigned ntile = (unsigned)(max_obj / 1024 + 1);
-    k_clean_count<<<ntile, 1024, 0, s>>>(n_dev, max_obj, w);
+    ipp_launch_dep(k_clean_count, dim3(ntile), 1024, 0, s, n_dev, max_obj, w);
     if (int e = ipp_check_launch("k_clean_count")) return e;
-    k_clean_assign<<<ntile, 1024, 0, s>>>(n_dev, max_obj, w, n_out);
+    ipp_launch_dep(k_clean_assign, dim3(ntile), 1024, 0, s, n_dev, max_obj, w, n_out);
     if (int e = ipp_check_launch("k_clean_assign")) return e;
-    k_clean_relabel<<<pg, CL_T, 0, s>>>(labels, npx, n_dev, max_obj, w, out);
+    ipp_launch_dep(k_clean_relabel, dim3(pg), CL_T, 0, s, labels, npx, n_dev, max_obj, w, out);
     return ipp_check_launch("k_clean_relabel");
 }

@@ -420,6 +420,7 @@ __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const fl
 // Candidates in region order (row-major over the regions) and their count.
 __global__ void __launch_bounds__(1024) k_sub_compact(const int2* reg, int nreg, int32_t* cx, int32_t* cy,
                                                       int32_t* n_dev) {
+    dep_begin();
     __shared__ int red[32];
     __shared__ int carry;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -494,6 +495,7 @@ __device__ void sub_terms_dev(double x, double y, int64_t W, int64_t H, int orde
 // [f0, f1) -- a cut of about equal work -- and the basis functions built on them.
 // 100 candidates on 152 SMs: 200 -> 173 us with three parts each.
 __global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J, int parts) {
+    dep_begin();
     extern __shared__ double sm[];
     const int c = blockIdx.x / parts, part = blockIdx.x - c * parts;
     if (c >= min(*J.n_dev, J.max_c)) return;
@@ -570,6 +572,7 @@ __global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J, int parts) {
 // cut into `parts` blocks in the same way: each takes an equal run of
 // the sums.  100 candidates: 180 -> 138 us.
 __global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J, int parts) {
+    dep_begin();
     extern __shared__ double sm[];
     const int c = blockIdx.x / parts, part = blockIdx.x - c * parts;
     if (c >= min(*J.n_dev, J.max_c)) return;
@@ -636,6 +639,7 @@ __global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J, int parts) {
 // AtA and Atb from the candidates' parts, summed in candidate order: one thread
 // per entry of the lower triangle (both halves written)
 __global__ void __launch_bounds__(256) k_sub_assemble(SubFitJob J) {
+    dep_begin();
     const int nc = min(*J.n_dev, J.max_c);
     const int np = J.np, nk = J.nb * J.ns, ns = J.ns, nb = J.nb, ng = J.ng;
     const int ntri = np * (np + 1) / 2;
@@ -684,7 +688,10 @@ __global__ void __launch_bounds__(256) k_sub_assemble(SubFitJob J) {
 // positive sets *status = 1; the later kernels then leave everything as is.
 constexpr int CB = 32;
 
-__global__ void k_chol_init(int32_t* status) { *status = 0; }
+__global__ void k_chol_init(int32_t* status) {
+    dep_begin();
+    *status = 0;
+}
 
 // The diagonal block.  Bound by the chain square root -> reciprocal -> scaled
 // column -> next pivot, so warp 0 runs that chain alone, one column ahead: it
@@ -694,6 +701,7 @@ __global__ void k_chol_init(int32_t* status) { *status = 0; }
 constexpr int CD_T = 256, CD_W = CD_T / 32;
 
 __global__ void __launch_bounds__(CD_T) k_chol_diag(double* A, int n, int k0, int32_t* status) {
+    dep_begin();
     __shared__ double D[CB][CB + 1];
     if (__ldcg(status)) return;
     const int b = min(CB, n - k0), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -765,6 +773,7 @@ __device__ __forceinline__ double div_by_recip(double a, double b, double y) {
 constexpr int CT_T = 64;
 
 __global__ void __launch_bounds__(CT_T) k_chol_trsm(double* A, int n, int k0, const int32_t* status) {
+    dep_begin();
     __shared__ double L[CB][CB + 1];
     if (__ldcg(status)) return;
     const int b = min(CB, n - k0);
@@ -794,6 +803,7 @@ __global__ void __launch_bounds__(CT_T) k_chol_trsm(double* A, int n, int k0, co
 constexpr int CS = 16;
 
 __global__ void __launch_bounds__(CS * CS) k_chol_syrk(double* A, int n, int k0, const int32_t* status) {
+    dep_begin();
     __shared__ double Li[CS][CB + 1], Lc[CS][CB + 1];
     if (__ldcg(status)) return;
     const int r0 = k0 + CB;
@@ -834,6 +844,7 @@ __device__ __forceinline__ void chol_stage_block(const double* A, int n, int r0,
 
 __global__ void __launch_bounds__(1024) k_chol_solve(const double* A, double* b, int n, double* x64, float* x32,
                                                      const int32_t* status) {
+    dep_begin();
     __shared__ double part[CB], rd[CB];
     __shared__ double Ld[CB][CB + 1];
     if (__ldcg(status)) return;
@@ -1001,7 +1012,7 @@ int ipp_launch_sub_stamps(const float* I, const float* R, int64_t W, int64_t H, 
     if (cudaLaunchKernelEx(&cfg, fn, I, R, W, H, pitch, nsx, nsy, hw, fh, nsig, slice, reg) != cudaSuccess)
         return ipp_check_launch("k_sub_stamps");
     if (int e = ipp_check_launch("k_sub_stamps")) return e;
-    k_sub_compact<<<1, 1024, 0, s>>>(reg, nsx * nsy, cx, cy, n_dev);
+    ipp_launch_dep(k_sub_compact, dim3(1), 1024, 0, s, reg, nsx * nsy, cx, cy, n_dev);
     return ipp_check_launch("k_sub_compact");
 }
 
@@ -1024,31 +1035,31 @@ int ipp_launch_sub_normal(const float* I, const float* R, int64_t W, int64_t H, 
     cudaFuncSetAttribute(k_sub_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.conv_smem);
     cudaFuncSetAttribute(k_sub_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.gram_smem);
     const int parts = sub_parts(max_c);
-    k_sub_conv<<<(unsigned)(max_c * parts), 256, d.conv_smem, s>>>(J, parts);
+    ipp_launch_dep(k_sub_conv, dim3((unsigned)(max_c * parts)), 256, d.conv_smem, s, J, parts);
     if (int e = ipp_check_launch("k_sub_conv")) return e;
-    k_sub_gram<<<(unsigned)(max_c * parts), 256, d.gram_smem, s>>>(J, parts);
+    ipp_launch_dep(k_sub_gram, dim3((unsigned)(max_c * parts)), 256, d.gram_smem, s, J, parts);
     if (int e = ipp_check_launch("k_sub_gram")) return e;
     const int nt = d.np * (d.np + 1) / 2 + d.np;
-    k_sub_assemble<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(J);
+    ipp_launch_dep(k_sub_assemble, dim3((unsigned)((nt + 255) / 256)), 256, 0, s, J);
     return ipp_check_launch("k_sub_assemble");
 }
 
 int ipp_launch_sub_solve(double* AtA, double* Atb, int np, double* coef64, float* coef, int32_t* status,
                          cudaStream_t s) {
-    k_chol_init<<<1, 1, 0, s>>>(status);
+    ipp_launch_dep(k_chol_init, dim3(1), 1, 0, s, status);
     if (int e = ipp_check_launch("k_chol_init")) return e;
     for (int k0 = 0; k0 < np; k0 += CB) {
-        k_chol_diag<<<1, CD_T, 0, s>>>(AtA, np, k0, status);
+        ipp_launch_dep(k_chol_diag, dim3(1), CD_T, 0, s, AtA, np, k0, status);
         if (int e = ipp_check_launch("k_chol_diag")) return e;
         const int rest = np - k0 - CB;
         if (rest <= 0) break;
-        k_chol_trsm<<<(unsigned)((rest + CT_T / 32 - 1) / (CT_T / 32)), CT_T, 0, s>>>(AtA, np, k0, status);
+        ipp_launch_dep(k_chol_trsm, dim3((unsigned)((rest + CT_T / 32 - 1) / (CT_T / 32))), CT_T, 0, s, AtA, np, k0, status);
         if (int e = ipp_check_launch("k_chol_trsm")) return e;
         const int nt = (rest + CS - 1) / CS;
-        k_chol_syrk<<<(unsigned)(nt * (nt + 1) / 2), CS * CS, 0, s>>>(AtA, np, k0, status);
+        ipp_launch_dep(k_chol_syrk, dim3((unsigned)(nt * (nt + 1) / 2)), CS * CS, 0, s, AtA, np, k0, status);
         if (int e = ipp_check_launch("k_chol_syrk")) return e;
     }
-    k_chol_solve<<<1, 1024, 0, s>>>(AtA, Atb, np, coef64, coef, status);
+    ipp_launch_dep(k_chol_solve, dim3(1), 1024, 0, s, AtA, Atb, np, coef64, coef, status);
     return ipp_check_launch("k_chol_solve");
 }
 
