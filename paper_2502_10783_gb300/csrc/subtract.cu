@@ -15,7 +15,7 @@
 // multiply-adds costs C + 2 hw + 3 S / 4 shared loads: bound by the FP32 pipe
 // instead of shared memory.  Per output the sum still runs over the kernel's rows,
 // then columns, in ascending order.  4096 x 4096, hw = 10, 49 basis functions:
-// 767 -> 532 us (one row of 7 outputs a thread, before); the convolution's
+// 767 -> 473 us (one row of 7 outputs a thread, before); the convolution's
 // 7.4 G multiply-adds alone are 191 us of this part's FP32 rate.
 #include <math.h>
 
@@ -102,6 +102,8 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
     const int64_t bx = blockIdx.x % ntx, by = blockIdx.x / ntx;
     const int64_t x0 = bx * (S * TPB), y0 = by * S;
     const float sx = W > 1 ? 2.f / (float)(W - 1) : 0.f, sy = H > 1 ? 2.f / (float)(H - 1) : 0.f;
+    // background terms 1, y, x of the usual order, read before they are needed
+    const float cb0 = bord == 1 ? __ldg(cb) : 0.f, cb1 = bord == 1 ? __ldg(cb + 1) : 0.f, cb2 = bord == 1 ? __ldg(cb + 2) : 0.f;
     // Eq. 8 at the tiles' centres
     for (int t = threadIdx.x; t < TPB * nb; t += T) {
         const int tile = t / nb, n = t - tile * nb;
@@ -116,11 +118,21 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
     }
     // template window: rows y0 - HW .., columns x0 - HW .. (0 outside the frame and
     // in the rows and columns that only padding outputs read)
-    for (int t = threadIdx.x; t < SH::WROWS * SH::WCOLS; t += T) {
-        const int a = t / SH::WCOLS, b = t - a * SH::WCOLS;
-        const int64_t yy = y0 - HW + a, xx = x0 - HW + b;
-        const bool in = a < S + 2 * HW && b < S * TPB + 2 * HW && yy >= 0 && yy < H && xx >= 0 && xx < W;
-        Rw[a * WP + b] = in ? __ldg(R + yy * pitch + xx) : 0.f;
+    constexpr int NWIN = SH::WROWS * SH::WCOLS, LB = 9;   // LB loads in flight a thread
+    for (int t0 = threadIdx.x; t0 < NWIN; t0 += LB * T) {
+        float v[LB];
+#pragma unroll
+        for (int m = 0; m < LB; m++) {
+            const int t = t0 + m * T, a = t / SH::WCOLS, b = t - a * SH::WCOLS;
+            const int64_t yy = y0 - HW + a, xx = x0 - HW + b;
+            const bool in = a < S + 2 * HW && b < S * TPB + 2 * HW && yy >= 0 && yy < H && xx >= 0 && xx < W;
+            v[m] = in ? __ldg(R + yy * pitch + xx) : 0.f;
+        }
+#pragma unroll
+        for (int m = 0; m < LB; m++) {
+            const int t = t0 + m * T, a = t / SH::WCOLS;
+            if (t < NWIN) Rw[a * WP + t - a * SH::WCOLS] = v[m];
+        }
     }
     __syncthreads();
     // Eq. 9 summed with the tiles' amplitudes: one read of a basis value (from L2)
@@ -197,17 +209,28 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
         for (int q = 0; q < C; q++)
             if (oy0 + r < S && ox0 + q < S) Rw[(oy0 + r) * (S * TPB) + tile * S + ox0 + q] = acc[r][q];
     __syncthreads();
-    for (int t = threadIdx.x; t < S * S * TPB; t += T) {
-        const int oy = t / (S * TPB), ox = t - oy * (S * TPB);
-        const int64_t x = x0 + ox, y = y0 + oy;
-        if (x >= W || y >= H) continue;
-        float r = NAN;
-        if (x >= HW && y >= HW && x <= W - 1 - HW && y <= H - 1 - HW) {
+    // the difference, EB pixels of the frame in flight a thread
+    constexpr int NOUT = S * S * TPB, EB = 7;
+    for (int t0 = threadIdx.x; t0 < NOUT; t0 += EB * T) {
+        float v[EB];
+#pragma unroll
+        for (int m = 0; m < EB; m++) {
+            const int t = t0 + m * T, oy = t / (S * TPB), ox = t - oy * (S * TPB);
+            const int64_t x = x0 + ox, y = y0 + oy;
+            v[m] = t < NOUT && x >= HW && y >= HW && x <= W - 1 - HW && y <= H - 1 - HW ? __ldg(I + y * pitch + x) : NAN;
+        }
+#pragma unroll
+        for (int m = 0; m < EB; m++) {
+            const int t = t0 + m * T, oy = t / (S * TPB), ox = t - oy * (S * TPB);
+            const int64_t x = x0 + ox, y = y0 + oy;
+            if (t >= NOUT || x >= W || y >= H) continue;
             float b = 0.f;
-            if (bord >= 0) {
-                // the terms of sub_terms in turn, without a table
-                const float xs = W > 1 ? (float)x * sx - 1.f : 0.f;
-                const float ys = H > 1 ? (float)y * sy - 1.f : 0.f;
+            // the terms of sub_terms in turn, without a table
+            const float xs = W > 1 ? (float)x * sx - 1.f : 0.f;
+            const float ys = H > 1 ? (float)y * sy - 1.f : 0.f;
+            if (bord == 1) {
+                b = fmaf(cb2, xs, fmaf(cb1, ys, cb0));
+            } else {
                 const float* c = cb;
                 float xp = 1.f;
                 for (int p = 0; p <= bord; p++) {
@@ -219,9 +242,10 @@ __global__ void __launch_bounds__(SubApplyShape<HW, C, TPB, WP>::T)
                     xp *= xs;
                 }
             }
-            r = __ldg(I + y * pitch + x) + b - Rw[t];
+            // pixels whose support leaves the frame stay NaN
+            const bool in = x >= HW && y >= HW && x <= W - 1 - HW && y <= H - 1 - HW;
+            D[y * opitch + x] = in ? v[m] + b - Rw[t] : NAN;
         }
-        D[y * opitch + x] = r;
     }
 }
 
