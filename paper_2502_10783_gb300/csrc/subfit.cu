@@ -637,7 +637,24 @@ __global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J, int parts) {
 }
 
 // AtA and Atb from the candidates' parts, summed in candidate order: one thread
-// per entry of the lower triangle (both halves written)
+// per entry of the lower triangle (both halves written).  Bound by latency: a
+// candidate's parts lie apart, so eight candidates' loads are issued before their
+// sums are formed.  100 candidates, 297 unknowns: 50 -> 40 us.
+template <class Load, class Term>
+__device__ __forceinline__ double sum_candidates(int nc, Load&& load, Term&& term) {
+    constexpr int B = 8;
+    double s = 0.0;
+    for (int c0 = 0; c0 < nc; c0 += B) {
+        double v[B][3];
+#pragma unroll
+        for (int q = 0; q < B; q++) load(min(c0 + q, nc - 1), v[q]);
+#pragma unroll
+        for (int q = 0; q < B; q++)
+            if (c0 + q < nc) term(s, v[q]);
+    }
+    return s;
+}
+
 __global__ void __launch_bounds__(256) k_sub_assemble(SubFitJob J) {
     dep_begin();
     const int nc = min(*J.n_dev, J.max_c);
@@ -661,18 +678,32 @@ __global__ void __launch_bounds__(256) k_sub_assemble(SubFitJob J) {
         while (a * (a + 1) / 2 > t) a--;
         while ((a + 1) * (a + 2) / 2 <= t) a++;
         const int b = t - a * (a + 1) / 2;                 // b <= a
-        double s = 0.0;
+        double s;
         if (a < nk) {                                      // both kernel unknowns
             const int n = a / ns, sa = a - n * ns, mm = b / ns, sb = b - mm * ns;
             const int hi = max(n, mm), lo = min(n, mm);
-            for (int c = 0; c < nc; c++)
-                s += J.Ps[(size_t)c * ns + sa] * J.Ps[(size_t)c * ns + sb] * J.G[((size_t)c * nb + hi) * nb + lo];
+            s = sum_candidates(
+                nc,
+                [&](int c, double* v) {
+                    v[0] = J.Ps[(size_t)c * ns + sa];
+                    v[1] = J.Ps[(size_t)c * ns + sb];
+                    v[2] = J.G[((size_t)c * nb + hi) * nb + lo];
+                },
+                [](double& t, const double* v) { t += v[0] * v[1] * v[2]; });
         } else if (b < nk) {                               // background row a, kernel column b
             const int g = a - nk, mm = b / ns, sb = b - mm * ns;
-            for (int c = 0; c < nc; c++) s -= J.Ps[(size_t)c * ns + sb] * J.X[((size_t)c * nb + mm) * ng + g];
+            s = sum_candidates(
+                nc,
+                [&](int c, double* v) {
+                    v[0] = J.Ps[(size_t)c * ns + sb];
+                    v[1] = J.X[((size_t)c * nb + mm) * ng + g];
+                },
+                [](double& t, const double* v) { t -= v[0] * v[1]; });
         } else {                                           // both background
             const int g = a - nk, hh = b - nk;
-            for (int c = 0; c < nc; c++) s += J.BB[((size_t)c * ng + g) * ng + hh];
+            s = sum_candidates(
+                nc, [&](int c, double* v) { v[0] = J.BB[((size_t)c * ng + g) * ng + hh]; },
+                [](double& t, const double* v) { t += v[0]; });
         }
         J.AtA[(size_t)a * np + b] = s;
         J.AtA[(size_t)b * np + a] = s;
