@@ -181,7 +181,7 @@ __device__ __forceinline__ float div_fast(float a, float b) {
     return y;
 }
 
-// chi^2, J'WJ and J'Wr of one stamp at pp.  The model of psf_eval with the
+// chi^2, J'WJ and J'Wr of one stamp at pp.  The model of k_psf_fwd with the
 // per-trial constants (reciprocal widths, normalisation, trig) taken out of the
 // pixel loop and its derivatives regrouped around T = 2 dP/dq, a = u/sx^2 and
 // b = v/sy^2:
