@@ -378,80 +378,80 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ sr
     const int Wi = (int)W, Hi = (int)H;
     for (int64_t t0 = ((int64_t)blockIdx.x * (AL_T / 32) + (threadIdx.x >> 5)) * RP_GRP; t0 < tasks;
          t0 += warps * RP_GRP) {
-      // lane l: segment t0 + l's row, first column and source position
-      int mi = 0, mj = 0, mbx = 0, mby = 0, mok = 0;
-      float mfx = 0.f, mfy = 0.f;
-      if (lane < RP_GRP && t0 + lane < tasks) {
-        const int64_t i = (t0 + lane) / segs, j0 = (t0 + lane - i * segs) * RP_SEG;
-        // first source position of the segment, Minv (j0, i, 1), in double-float
-        const float fj = (float)(int)j0, fi = (float)(int)i;   // exact: Wo, Ho < 2^24
-        const df X0 = df_add(df_add(df_mul_exact(m0, fj), df_mul_exact(m1, fi)), m2);
-        const df Y0 = df_add(df_add(df_mul_exact(m3, fj), df_mul_exact(m4, fi)), m5);
-        const bool base_ok = sane && fabsf(X0.hi) < lim && fabsf(Y0.hi) < lim;
-        int ibx = 0, iby = 0;
-        float fbx = 0.f, fby = 0.f;
-        if (base_ok) {
-            df_floor(X0, ibx, fbx);
-            df_floor(Y0, iby, fby);
-        }
-        // the positions are monotone along the segment: when both ends have all four
-        // neighbours inside the frame, so has every pixel between (no per-pixel
-        // bounds tests, four unconditional loads)
-        const int kmax = (int)min((int64_t)RP_SEG, Wo - j0) - 1;
-        bool interior = false;
-        if (base_ok) {
-            const float xb = fmaf(f0, (float)kmax, fbx), yb = fmaf(f3, (float)kmax, fby);
-            const int ixa = ibx + (int)floorf(fbx), ixb = ibx + (int)floorf(xb);
-            const int iya = iby + (int)floorf(fby), iyb = iby + (int)floorf(yb);
-            interior = min(ixa, ixb) >= 0 && max(ixa, ixb) <= Wi - 2 && min(iya, iyb) >= 0 && max(iya, iyb) <= Hi - 2;
-        }
-        mi = (int)i; mj = (int)j0; mbx = ibx; mby = iby; mfx = fbx; mfy = fby;
-        mok = (base_ok ? 1 : 0) | (interior ? 2 : 0);
-      }
-      const int nseg = (int)min((int64_t)RP_GRP, tasks - t0);
-      for (int g = 0; g < nseg; g++) {
-        const int64_t i = __shfl_sync(0xffffffffu, mi, g), j0 = __shfl_sync(0xffffffffu, mj, g);
-        const int ibx = __shfl_sync(0xffffffffu, mbx, g), iby = __shfl_sync(0xffffffffu, mby, g);
-        const float fbx = __shfl_sync(0xffffffffu, mfx, g), fby = __shfl_sync(0xffffffffu, mfy, g);
-        const int ok = __shfl_sync(0xffffffffu, mok, g);
-        const bool base_ok = ok & 1, interior = ok & 2;
-        const int kmax = (int)min((int64_t)RP_SEG, Wo - j0) - 1;
-        float v[4];
-#pragma unroll
-        for (int c = 0; c < 4; c++) {
-            const int k = lane * 4 + c;
-            float r = fill;
-            if (base_ok && k <= kmax) {
-                const float fx = fmaf(f0, (float)k, fbx), fy = fmaf(f3, (float)k, fby);
-                const float flx = floorf(fx), fly = floorf(fy);
-                const int ix = ibx + (int)flx, iy = iby + (int)fly;
-                const float tx = fx - flx, ty = fy - fly;
-                if (interior) {
-                    const float* row = src + (int64_t)iy * pitch + ix;
-                    const float q00 = __ldg(row), q10 = __ldg(row + 1);
-                    const float q01 = __ldg(row + pitch), q11 = __ldg(row + pitch + 1);
-                    const float w00 = (1.f - tx) * (1.f - ty), w10 = tx * (1.f - ty), w01 = (1.f - tx) * ty,
-                                w11 = tx * ty;
-                    // the same sum, in the same order, as the careful form: a term of
-                    // zero weight adds 0 exactly when its value is finite
-                    const float acc = fmaf(w11, q11, fmaf(w01, q01, fmaf(w10, q10, w00 * q00)));
-                    r = isfinite(acc) ? acc : rp_careful(src, pitch, Wi, Hi, ix, iy, tx, ty, fill);
-                } else {
-                    r = rp_careful(src, pitch, Wi, Hi, ix, iy, tx, ty, fill);
-                }
+        // lane l: segment t0 + l's row, first column and source position
+        int mi = 0, mj = 0, mbx = 0, mby = 0, mok = 0;
+        float mfx = 0.f, mfy = 0.f;
+        if (lane < RP_GRP && t0 + lane < tasks) {
+            const int64_t i = (t0 + lane) / segs, j0 = (t0 + lane - i * segs) * RP_SEG;
+            // first source position of the segment, Minv (j0, i, 1), in double-float
+            const float fj = (float)(int)j0, fi = (float)(int)i;   // exact: Wo, Ho < 2^24
+            const df X0 = df_add(df_add(df_mul_exact(m0, fj), df_mul_exact(m1, fi)), m2);
+            const df Y0 = df_add(df_add(df_mul_exact(m3, fj), df_mul_exact(m4, fi)), m5);
+            const bool base_ok = sane && fabsf(X0.hi) < lim && fabsf(Y0.hi) < lim;
+            int ibx = 0, iby = 0;
+            float fbx = 0.f, fby = 0.f;
+            if (base_ok) {
+                df_floor(X0, ibx, fbx);
+                df_floor(Y0, iby, fby);
             }
-            v[c] = r;
+            // the positions are monotone along the segment: when both ends have all four
+            // neighbours inside the frame, so has every pixel between (no per-pixel
+            // bounds tests, four unconditional loads)
+            const int kmax = (int)min((int64_t)RP_SEG, Wo - j0) - 1;
+            bool interior = false;
+            if (base_ok) {
+                const float xb = fmaf(f0, (float)kmax, fbx), yb = fmaf(f3, (float)kmax, fby);
+                const int ixa = ibx + (int)floorf(fbx), ixb = ibx + (int)floorf(xb);
+                const int iya = iby + (int)floorf(fby), iyb = iby + (int)floorf(yb);
+                interior = min(ixa, ixb) >= 0 && max(ixa, ixb) <= Wi - 2 && min(iya, iyb) >= 0 && max(iya, iyb) <= Hi - 2;
+            }
+            mi = (int)i; mj = (int)j0; mbx = ibx; mby = iby; mfx = fbx; mfy = fby;
+            mok = (base_ok ? 1 : 0) | (interior ? 2 : 0);
         }
-        const int64_t jj = j0 + lane * 4;
-        float* orow = out + i * opitch;
-        if (vout && jj + 4 <= Wo) {
-            *reinterpret_cast<float4*>(orow + jj) = make_float4(v[0], v[1], v[2], v[3]);
-        } else {
+        const int nseg = (int)min((int64_t)RP_GRP, tasks - t0);
+        for (int g = 0; g < nseg; g++) {
+            const int64_t i = __shfl_sync(0xffffffffu, mi, g), j0 = __shfl_sync(0xffffffffu, mj, g);
+            const int ibx = __shfl_sync(0xffffffffu, mbx, g), iby = __shfl_sync(0xffffffffu, mby, g);
+            const float fbx = __shfl_sync(0xffffffffu, mfx, g), fby = __shfl_sync(0xffffffffu, mfy, g);
+            const int ok = __shfl_sync(0xffffffffu, mok, g);
+            const bool base_ok = ok & 1, interior = ok & 2;
+            const int kmax = (int)min((int64_t)RP_SEG, Wo - j0) - 1;
+            float v[4];
 #pragma unroll
-            for (int c = 0; c < 4; c++)
-                if (jj + c < Wo) orow[jj + c] = v[c];
+            for (int c = 0; c < 4; c++) {
+                const int k = lane * 4 + c;
+                float r = fill;
+                if (base_ok && k <= kmax) {
+                    const float fx = fmaf(f0, (float)k, fbx), fy = fmaf(f3, (float)k, fby);
+                    const float flx = floorf(fx), fly = floorf(fy);
+                    const int ix = ibx + (int)flx, iy = iby + (int)fly;
+                    const float tx = fx - flx, ty = fy - fly;
+                    if (interior) {
+                        const float* row = src + (int64_t)iy * pitch + ix;
+                        const float q00 = __ldg(row), q10 = __ldg(row + 1);
+                        const float q01 = __ldg(row + pitch), q11 = __ldg(row + pitch + 1);
+                        const float w00 = (1.f - tx) * (1.f - ty), w10 = tx * (1.f - ty), w01 = (1.f - tx) * ty,
+                                    w11 = tx * ty;
+                        // the same sum, in the same order, as the careful form: a term of
+                        // zero weight adds 0 exactly when its value is finite
+                        const float acc = fmaf(w11, q11, fmaf(w01, q01, fmaf(w10, q10, w00 * q00)));
+                        r = isfinite(acc) ? acc : rp_careful(src, pitch, Wi, Hi, ix, iy, tx, ty, fill);
+                    } else {
+                        r = rp_careful(src, pitch, Wi, Hi, ix, iy, tx, ty, fill);
+                    }
+                }
+                v[c] = r;
+            }
+            const int64_t jj = j0 + lane * 4;
+            float* orow = out + i * opitch;
+            if (vout && jj + 4 <= Wo) {
+                *reinterpret_cast<float4*>(orow + jj) = make_float4(v[0], v[1], v[2], v[3]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; c++)
+                    if (jj + c < Wo) orow[jj + c] = v[c];
+            }
         }
-      }
     }
 }
 
