@@ -221,3 +221,41 @@ def test_extract_repeats(gpu, W, H, mesh):
         assert torch.equal(ex.out["labels"], ref["labels"]) and torch.equal(ex.out["sub"], ref["sub"])
         for k in ("x", "y", "flux", "sky"):
             assert torch.equal(ex.out[k][:n], ref[k][:n])
+
+
+# Kron apertures whose box gives a thread 16 pixels a row and more (rows told apart by two
+# bounds) and narrower ones, for footprints above and below the block form's 128
+# pixels, inside and beyond the frame.
+# The moments are FP32 sums (1e-4 relative), so the ellipse's area may differ by 1e-3 of
+# itself; one that holds the frame holds every pixel.
+@pytest.mark.parametrize("k_kron", [12.0, 25.0, 60.0, 1e4])
+def test_wide_kron_apertures(gpu, orc, k_kron):
+    H, W = 120, 4203
+    rng = np.random.default_rng(3)
+    yy, xx = np.mgrid[:H, :W]
+    sub = rng.normal(0.0, 1.0, (H, W))
+    lab = np.zeros((H, W), np.int32)
+    stats = {k: [] for k in ("xmin", "xmax", "ymin", "ymax", "xbar", "ybar")}
+    for n, (cx, cy, a, b, th) in enumerate([(2000, 50, 2.0, 1.6, 0.0), (900, 60, 5.0, 1.5, 0.1), (3300, 70, 9.0, 2.0, -0.05),
+                                            (8, 100, 3.0, 2.5, 0.3)]):
+        u = (xx - cx) * np.cos(th) + (yy - cy) * np.sin(th)
+        v = (yy - cy) * np.cos(th) - (xx - cx) * np.sin(th)
+        q = (u / a) ** 2 + (v / b) ** 2
+        sub += 200.0 * np.exp(-0.5 * q)
+        foot = (q < 5.0) & (lab == 0)
+        lab[foot] = n + 1
+        for k, m in (("xmin", xx[foot].min()), ("xmax", xx[foot].max()), ("ymin", yy[foot].min()), ("ymax", yy[foot].max()),
+                     ("xbar", cx + 0.25), ("ybar", cy - 0.125)):
+            stats[k].append(m)
+    sub = sub.astype(np.float32)
+    st = {k: np.asarray(v, np.float32 if k[1:] == "bar" else np.int32) for k, v in stats.items()}
+    o = orc.auto_phot(sub, lab, st, k_kron=k_kron)
+    full = gpu._alloc_stats(4, torch.device("cuda"))
+    for k, v in st.items():
+        full[k].copy_(dev(v))
+    g = gpu.auto_phot(dev(sub), dev(lab), torch.tensor([4], dtype=torch.int32, device="cuda"), full, k_kron=k_kron)
+    g = {k: host(v) for k, v in g.items()}
+    assert np.array_equal(g["flags"], o["flags"])
+    edge = np.where(o["area"] == W * H, 0.0, 1e-3 * o["area"] + 4.0)
+    assert np.all(np.abs(g["area"] - o["area"]) <= edge)
+    assert np.all(np.abs(g["flux"] - o["flux"]) <= 1e-5 * np.abs(sub).sum() + 6.0 * edge)
