@@ -32,9 +32,11 @@ constexpr int T_CAP = (T_TH / 2) * (T_TW / 2);   // max 8-connected components i
 constexpr int T_RCAP = T_TH * (T_TW / 2);        // max runs in a tile
 constexpr int T_THREADS = 128;
 // tile kernel capacities: the common pass keeps up to 1024 runs (and the stats
-// of 128 kept components) in shared memory, so ten tiles fit on an SM; tiles
-// with more runs are redone by a second pass with the full capacity
-constexpr int T_RCAP_FAST = 1024, KCAP_FAST = 128;
+// of 96 kept components, four times what a survey frame's tiles hold) in 21.5 KB of
+// shared memory, so ten tiles fit on an SM; tiles with more runs are redone by a
+// second pass with the full capacity.  128 components leave nine tiles an SM (63
+// against 61 us on a 4096 x 4096 frame)
+constexpr int T_RCAP_FAST = 1024, KCAP_FAST = 96;
 constexpr int KCAP_FULL = 256;
 constexpr int T_NQ = 40;
 
@@ -58,7 +60,7 @@ struct CclWs {
     int32_t* label;
     int32_t* btop; int32_t* bbot;    // [ntiles*T_TW]
     int32_t* blef; int32_t* brig;    // [ntiles*T_TH]
-    int32_t* counters;   // [0] kept nodes listed, [1] overflow tiles (zeroed by the host before the tile pass)
+    int32_t* counters;   // [0] kept nodes listed, [1] overflow tiles (zeroed before the tile pass)
     int32_t* trcnt;      // [nty] surviving components per tile row (zeroed with counters)
     int32_t* klist;      // [ntiles*T_CAP] kept node ids, in no particular order
     int32_t* lpos;       // [nodes] tile-local index (row * T_TW + col) of the node's own first pixel
