@@ -609,7 +609,7 @@ def main():
     # (49 x 441 multiply-adds a tile); FP32 ALU-bound
     sub_flops = 2.0 * 441 * W * H + 2.0 * 49 * 441 * ((W + 20) // 21) * ((H + 20) // 21)
     subtraction = {"ms": stages["sub_apply"], "achieved_tflops": sub_flops / (stages["sub_apply"] / 1e3) / 1e12,
-                   "flops_per_call": sub_flops, "kernels": "k_sub_basis + k_sub_apply (one block per 21 x 21 tile)",
+                   "flops_per_call": sub_flops, "kernels": "k_sub_basis + k_sub_apply (a block per three 21 x 21 tiles)",
                    "workload": "survey_4k subtracted frame against a copy, 21 x 21 kernel, 49 basis functions",
                    "fit_ms": stages["sub_fit"], "fit_status": sub_fit_status,
                    "fit_kernels": "k_sub_stamps + k_sub_compact + k_sub_conv + k_sub_gram + k_sub_assemble + "
@@ -618,7 +618,7 @@ def main():
     gb = 8 * W * H / (stages["reproject"] / 1e3) / 1e9
     align = {"ms": stages["align"], "reproject_ms": stages["reproject"], "reproject_bytes_per_px": 8,
              "reproject_achieved_gbs": gb, "reproject_frac_of_measured_hbm": gb / hbm,
-             "kernels": "k_wcs_map (32 px nodes, FP64) + k_aff_sum1/2 + k_aff_solve + k_reproject",
+             "kernels": "k_wcs_map (32 px nodes, FP64) + k_aff_sum1/2 + k_reproject",
              "workload": "survey_4k subtracted frame onto a second exposure's grid (pointing offset "
                          "0.02-0.05 deg, rotated, SIP order 3 on both)"}
 
