@@ -164,10 +164,12 @@ struct DistKeyD {
 // The k-th smallest key (0-based) of the region: radix selection, 8 bits a
 // pass from bit top + 7 down, every key sharing the bits above top with
 // prefix0; per-warp histograms in shared memory, fed by per-thread run lengths
-// of equal digits, summed over the block, then over the cluster.
+// of equal digits, summed over the block, then over the cluster.  A key known to be
+// `limit` or more after some digits ends the search (the caller has no use for it).
 template <class Key>
 __device__ unsigned long long region_select(StampRegion& g, const Key& key_of, long long k, int top,
-                                            unsigned long long prefix0, StampShared& S) {
+                                            unsigned long long prefix0, unsigned long long limit,
+                                            StampShared& S) {
     using T = typename Key::T;
     auto cl = cooperative_groups::this_cluster();
     T prefix = (T)prefix0;
@@ -235,6 +237,7 @@ __device__ unsigned long long region_select(StampRegion& g, const Key& key_of, l
         prefix = (T)(prefix << 8) | (T)S.sdig;
         k -= S.sbelow;
         __syncthreads();
+        if (((unsigned long long)prefix << shift) >= limit) return (unsigned long long)prefix << shift;
     }
     return prefix;
 }
@@ -244,14 +247,15 @@ __device__ unsigned long long region_select(StampRegion& g, const Key& key_of, l
 // and kmax differ
 template <class Key>
 __device__ void region_middle(StampRegion& g, const Key& key_of, long long n, unsigned long long kmin,
-                              unsigned long long kmax, StampShared& S, unsigned long long* a, unsigned long long* b) {
+                              unsigned long long kmax, unsigned long long limit, StampShared& S,
+                              unsigned long long* a, unsigned long long* b) {
     using T = typename Key::T;
     const long long k0 = (n - 1) / 2, k1 = n / 2;
     const unsigned long long dif = kmin ^ kmax;
     const int top = dif ? ((63 - __clzll((long long)dif)) & ~7) : 0;
     const unsigned long long prefix0 = top + 8 < 64 ? kmin >> (top + 8) : 0ull;
-    *a = region_select(g, key_of, k0, top, prefix0, S);
-    if (k1 == k0) { *b = *a; return; }
+    *a = region_select(g, key_of, k0, top, prefix0, limit, S);
+    if (k1 == k0 || *a >= limit) { *b = *a; return; }
     // count of keys <= a, smallest key > a
     uint32_t cnt = 0;
     T next = (T)~(T)0;
@@ -348,7 +352,7 @@ __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const fl
     }
     // median (Eq. 1's even-count mean of the middle pair)
     unsigned long long ka, kb;
-    region_middle(g, ValueKey{}, n, gmin, gmax, S, &ka, &kb);
+    region_middle(g, ValueKey{}, n, gmin, gmax, ~0ull, S, &ka, &kb);
     const double va = (double)fkey_inv((uint32_t)ka), vb = (double)fkey_inv((uint32_t)kb);
     const double med = (n & 1) ? vb : __dmul_rn(0.5, __dadd_rn(va, vb));
     // MAD: exact integer differences at scale 2^e0 when they fit 62 bits
@@ -365,14 +369,15 @@ __global__ void __launch_bounds__(SS_T, 2) k_sub_stamps(const float* I, const fl
         const long long exact32 = 2147483647ll - (imed < 0 ? -imed : imed);
         bool done = false;
         if (exact32 > 0) {
-            region_middle(g, DistKey32{s1, s2, (int)imed}, n, 0ull, top < 0xffffffffull ? top : 0xffffffffull, S, &ka, &kb);
+            region_middle(g, DistKey32{s1, s2, (int)imed}, n, 0ull, top < 0xffffffffull ? top : 0xffffffffull,
+                          (unsigned long long)exact32, S, &ka, &kb);
             done = (long long)kb < exact32;
         }
-        if (!done) region_middle(g, DistKey64{s1, s2, imed}, n, 0ull, top, S, &ka, &kb);
+        if (!done) region_middle(g, DistKey64{s1, s2, imed}, n, 0ull, top, ~0ull, S, &ka, &kb);
         da = ldexp((double)ka, e0);
         db = ldexp((double)kb, e0);
     } else {
-        region_middle(g, DistKeyD{med}, n, 0ull, ~0ull, S, &ka, &kb);
+        region_middle(g, DistKeyD{med}, n, 0ull, ~0ull, ~0ull, S, &ka, &kb);
         da = __longlong_as_double((long long)ka);
         db = __longlong_as_double((long long)kb);
     }
