@@ -325,8 +325,8 @@ __device__ __forceinline__ void df_floor(df a, int& ip, float& frac) {
 // one output pixel at source position (ix + tx, iy + ty): 0 <= x <= W - 1 and
 // 0 <= y <= H - 1, the pair beyond the last column / row not read, `fill` when
 // outside or when a neighbour of non-zero weight is not finite
-__device__ __forceinline__ float rp_careful(const float* __restrict__ src, int64_t pitch, int Wi, int Hi, int ix,
-                                           int iy, float tx, float ty, float fill) {
+__device__ __forceinline__ float rp_careful(const float* src, int64_t pitch, int Wi, int Hi, int ix, int iy,
+                                            float tx, float ty, float fill) {
     const bool in = ix >= 0 && iy >= 0 && (ix < Wi - 1 || (ix == Wi - 1 && tx == 0.f)) &&
                     (iy < Hi - 1 || (iy == Hi - 1 && ty == 0.f));
     if (!in) return fill;
@@ -337,15 +337,15 @@ __device__ __forceinline__ float rp_careful(const float* __restrict__ src, int64
     const float* row = src + (int64_t)y0 * pitch + x0;
     float acc = 0.f;
     bool bad = false;
-    if (w00 != 0.f) { const float q = __ldg(row); bad |= !isfinite(q); acc = fmaf(w00, q, acc); }
-    if (w10 != 0.f) { const float q = __ldg(row + 1); bad |= !isfinite(q); acc = fmaf(w10, q, acc); }
-    if (w01 != 0.f) { const float q = __ldg(row + pitch); bad |= !isfinite(q); acc = fmaf(w01, q, acc); }
-    if (w11 != 0.f) { const float q = __ldg(row + pitch + 1); bad |= !isfinite(q); acc = fmaf(w11, q, acc); }
+    if (w00 != 0.f) { const float q = dep_ld(row); bad |= !isfinite(q); acc = fmaf(w00, q, acc); }
+    if (w10 != 0.f) { const float q = dep_ld(row + 1); bad |= !isfinite(q); acc = fmaf(w10, q, acc); }
+    if (w01 != 0.f) { const float q = dep_ld(row + pitch); bad |= !isfinite(q); acc = fmaf(w01, q, acc); }
+    if (w11 != 0.f) { const float q = dep_ld(row + pitch + 1); bad |= !isfinite(q); acc = fmaf(w11, q, acc); }
     return bad ? fill : acc;
 }
 
-__global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ src, int64_t W, int64_t H,
-                                                    int64_t pitch, const double* __restrict__ Minv, int64_t Wo,
+__global__ void __launch_bounds__(AL_T) k_reproject(const float* src, int64_t W, int64_t H,
+                                                    int64_t pitch, const double* Minv, int64_t Wo,
                                                     int64_t Ho, float fill, float* __restrict__ out,
                                                     int64_t opitch, bool vout) {
     dep_begin();
@@ -428,8 +428,8 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* __restrict__ sr
                     const float tx = fx - flx, ty = fy - fly;
                     if (interior) {
                         const float* row = src + (int64_t)iy * pitch + ix;
-                        const float q00 = __ldg(row), q10 = __ldg(row + 1);
-                        const float q01 = __ldg(row + pitch), q11 = __ldg(row + pitch + 1);
+                        const float q00 = dep_ld(row), q10 = dep_ld(row + 1);
+                        const float q01 = dep_ld(row + pitch), q11 = dep_ld(row + pitch + 1);
                         const float w00 = (1.f - tx) * (1.f - ty), w10 = tx * (1.f - ty), w01 = (1.f - tx) * ty,
                                     w11 = tx * ty;
                         // the same sum, in the same order, as the careful form: a term of

@@ -98,11 +98,11 @@ __device__ __forceinline__ bool mesh_value_at(const GG& G, int r, int c, float* 
     const int64_t yy = G.y0 + r, xx = G.x0 + c;
     float x;
     if (GG::kind == MK_F32 || (GG::kind == MK_ANY && G.dtype == IPP_F32)) {
-        x = __ldg(reinterpret_cast<const float*>(G.img) + yy * G.pitch + xx);
+        x = dep_ld(reinterpret_cast<const float*>(G.img) + yy * G.pitch + xx);
     } else {
-        const float raw = (float)__ldg(reinterpret_cast<const uint16_t*>(G.img) + yy * G.pitch + xx);
-        const float b = G.bias_map ? __ldg(G.bias_map + yy * G.W + xx) : G.bias;
-        x = (raw - b) * __ldg(G.inv_flat + yy * G.W + xx);
+        const float raw = (float)dep_ld(reinterpret_cast<const uint16_t*>(G.img) + yy * G.pitch + xx);
+        const float b = G.bias_map ? dep_ld(G.bias_map + yy * G.W + xx) : G.bias;
+        x = (raw - b) * dep_ld(G.inv_flat + yy * G.W + xx);
     }
     *out = x;
     return !(G.mask && G.mask[yy * G.W + xx]) && isfinite(x);
@@ -137,9 +137,9 @@ __device__ __forceinline__ void mesh_for_each_u16(const MeshGeom& G, F& f) {
 #pragma unroll
         for (int j = 0; j < VCH; j++) {
             const int rr = min(r, G.he - 1);
-            q[j] = __ldg(raw + (int64_t)rr * p4 + c);
+            q[j] = dep_ld(raw + (int64_t)rr * p4 + c);
             at[j] = (int64_t)rr * w4 + c;
-            w[j] = __ldg(flat + at[j]);
+            w[j] = dep_ld(flat + at[j]);
             r += dr;
             c += dc;
             if (c >= qpr) { c -= qpr; r++; }
@@ -147,7 +147,7 @@ __device__ __forceinline__ void mesh_for_each_u16(const MeshGeom& G, F& f) {
 #pragma unroll
         for (int j = 0; j < VCH; j++) {
             if (e0 + j * T >= nq) continue;
-            const float4 b = bias ? __ldg(bias + at[j]) : make_float4(G.bias, G.bias, G.bias, G.bias);
+            const float4 b = bias ? dep_ld(bias + at[j]) : make_float4(G.bias, G.bias, G.bias, G.bias);
             const float x[4] = {((float)q[j].x - b.x) * w[j].x, ((float)q[j].y - b.y) * w[j].y,
                                 ((float)q[j].z - b.z) * w[j].z, ((float)q[j].w - b.w) * w[j].w};
 #pragma unroll
@@ -171,7 +171,7 @@ __device__ __forceinline__ void mesh_for_each(const GG& G, F&& f) {
             float4 q[VCH];
 #pragma unroll
             for (int j = 0; j < VCH; j++) {
-                q[j] = __ldg(base + (int64_t)min(r, G.he - 1) * p4 + c);
+                q[j] = dep_ld(base + (int64_t)min(r, G.he - 1) * p4 + c);
                 r += dr;
                 c += dc;
                 if (c >= qpr) { c -= qpr; r++; }

@@ -62,7 +62,7 @@ struct CleanThr {
 };
 
 __device__ __forceinline__ int clean_n(const int32_t* n_dev, int32_t max_obj) {
-    return max(0, min(__ldg(n_dev), max_obj));
+    return max(0, min(dep_ld(n_dev), max_obj));
 }
 
 __global__ void __launch_bounds__(CL_T) k_clean_pix_a(const float* sub, int64_t pitch, const int32_t* labels,
@@ -70,10 +70,10 @@ __global__ void __launch_bounds__(CL_T) k_clean_pix_a(const float* sub, int64_t 
                                                       CleanWs ws) {
     const int n = clean_n(n_dev, max_obj);
     for (int64_t p = (int64_t)blockIdx.x * CL_T + threadIdx.x; p < W * H; p += (int64_t)gridDim.x * CL_T) {
-        const int l = __ldg(labels + p);
+        const int l = dep_ld(labels + p);
         if (l <= 0 || l > n) continue;
         const int64_t y = p / W, x = p - y * W;
-        const float f = __ldg(sub + y * pitch + x);
+        const float f = dep_ld(sub + y * pitch + x);
         const unsigned long long key = ((unsigned long long)fkey(f) << 32) | (unsigned long long)(~(uint32_t)p);
         atomicMax(ws.pkey + l, key);
         atomicAdd(reinterpret_cast<unsigned long long*>(ws.cnt + 3 * l), 1ull);
@@ -136,10 +136,10 @@ __global__ void __launch_bounds__(CL_T) k_clean_pix_b(const float* sub, int64_t 
     dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int64_t p = (int64_t)blockIdx.x * CL_T + threadIdx.x; p < W * H; p += (int64_t)gridDim.x * CL_T) {
-        const int l = __ldg(labels + p);
+        const int l = dep_ld(labels + p);
         if (l <= 0 || l > n) continue;
         const int64_t y = p / W, x = p - y * W;
-        const float f = __ldg(sub + y * pitch + x);
+        const float f = dep_ld(sub + y * pitch + x);
         if (!(f > 0.f)) continue;
         const float4 g = ws.geo[l];
         const float2 lo = ws.blo[l];
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_pix_b(const float* sub, int64_t 
 // the detection threshold at pixel (x, y): max(k rms(x, y), thresh_abs), rms the
 // Keys interpolation of the mesh rms (nodes clamped at the grid's edges)
 __device__ float clean_thr_at(const CleanThr& T, int64_t x, int64_t y) {
-    if (T.map) return __ldg(T.map + y * T.W + x);
+    if (T.map) return dep_ld(T.map + y * T.W + x);
     if (!T.mesh_rms) return T.thresh_abs;
     const float u = ((float)x + 0.5f) / T.mesh_w - 0.5f, v = ((float)y + 0.5f) / T.mesh_h - 0.5f;
     const float qf = floorf(u), pf = floorf(v);
@@ -166,7 +166,7 @@ __device__ float clean_thr_at(const CleanThr& T, int64_t x, int64_t y) {
     for (int a = 0; a < 4; a++) {
         const int p = clampi(p0 - 1 + a, 0, T.ny - 1);
         float r = 0.f;
-        for (int b = 0; b < 4; b++) r = fmaf(wx[b], __ldg(T.mesh_rms + p * T.nx + clampi(q0 - 1 + b, 0, T.nx - 1)), r);
+        for (int b = 0; b < 4; b++) r = fmaf(wx[b], dep_ld(T.mesh_rms + p * T.nx + clampi(q0 - 1 + b, 0, T.nx - 1)), r);
         acc = fmaf(wy[a], r, acc);
     }
     return fmaxf(T.k * acc, T.thresh_abs);
@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_relabel(const int32_t* labels, i
     dep_begin();
     const int n = clean_n(n_dev, max_obj);
     for (int64_t p = (int64_t)blockIdx.x * CL_T + threadIdx.x; p < npx; p += (int64_t)gridDim.x * CL_T) {
-        const int l = __ldg(labels + p);
+        const int l = dep_ld(labels + p);
         out[p] = (l <= 0 || l > n) ? 0 : ws.into[ws.num[l]];   // the number of the object's kept root
     }
 }

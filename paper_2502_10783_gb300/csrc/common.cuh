@@ -166,6 +166,14 @@ IPP_D void dep_begin() {
     if (gridDim.x * gridDim.y <= 608u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// Loads of a kernel that starts with dep_begin(), whose blocks are resident while the
+// kernel before it, of this call or of the call before, may still be writing what it
+// reads: plain loads, ordered by the wait.  The read-only path (__ldg, or a const
+// __restrict__ parameter) is specified for memory that stays the same for the kernel's
+// whole lifetime.
+template <class T>
+IPP_D T dep_ld(const T* p) { return *p; }
+
 IPP_HD int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 IPP_HD int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 

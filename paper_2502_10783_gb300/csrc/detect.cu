@@ -148,10 +148,10 @@ __device__ __forceinline__ bool mbit(const SH& S, int r, int c) {
 }
 
 __device__ __forceinline__ float tile_load_pix(const SubThreshJob& J, int64_t y, int64_t x) {
-    if (J.dtype == IPP_F32) return __ldg(reinterpret_cast<const float*>(J.img) + y * J.pitch + x);
-    float raw = (float)__ldg(reinterpret_cast<const uint16_t*>(J.img) + y * J.pitch + x);
-    float b = J.bias_map ? __ldg(J.bias_map + y * J.W + x) : J.bias;
-    return (raw - b) * __ldg(J.inv_flat + y * J.W + x);
+    if (J.dtype == IPP_F32) return dep_ld(reinterpret_cast<const float*>(J.img) + y * J.pitch + x);
+    float raw = (float)dep_ld(reinterpret_cast<const uint16_t*>(J.img) + y * J.pitch + x);
+    float b = J.bias_map ? dep_ld(J.bias_map + y * J.W + x) : J.bias;
+    return (raw - b) * dep_ld(J.inv_flat + y * J.W + x);
 }
 
 template <class SH>
@@ -286,7 +286,7 @@ __device__ __forceinline__ void sub_thresh_body(const SubThreshJob& J, int bx, i
         if (y >= J.H || xc >= J.W) continue;
         if (J.fused) {
             if (vin && full4) {
-                const float4 t4 = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(J.img) + y * J.pitch + xc));
+                const float4 t4 = dep_ld(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(J.img) + y * J.pitch + xc));
                 f[q][0] = t4.x; f[q][1] = t4.y; f[q][2] = t4.z; f[q][3] = t4.w;
             } else {
 #pragma unroll
@@ -302,7 +302,7 @@ __device__ __forceinline__ void sub_thresh_body(const SubThreshJob& J, int bx, i
 #pragma unroll
                 for (int b = 0; b < 6; b++) {
                     const int64_t xx = xc - 1 + b;
-                    row[a][b] = (yy >= 0 && yy < J.H && xx >= 0 && xx < J.W) ? __ldg(J.sub + yy * J.sub_pitch + xx) : 0.f;
+                    row[a][b] = (yy >= 0 && yy < J.H && xx >= 0 && xx < J.W) ? dep_ld(J.sub + yy * J.sub_pitch + xx) : 0.f;
                 }
             }
             const float wy0 = y > 0 ? 1.f : 0.f, wy2 = y + 1 < J.H ? 1.f : 0.f;
@@ -319,11 +319,11 @@ __device__ __forceinline__ void sub_thresh_body(const SubThreshJob& J, int bx, i
             }
         } else {
             if (vsub && full4) {
-                const float4 t4 = __ldg(reinterpret_cast<const float4*>(J.sub + y * J.sub_pitch + xc));
+                const float4 t4 = dep_ld(reinterpret_cast<const float4*>(J.sub + y * J.sub_pitch + xc));
                 f[q][0] = t4.x; f[q][1] = t4.y; f[q][2] = t4.z; f[q][3] = t4.w;
             } else {
 #pragma unroll
-                for (int c = 0; c < 4; c++) f[q][c] = (xc + c < J.W) ? __ldg(J.sub + y * J.sub_pitch + xc + c) : 0.f;
+                for (int c = 0; c < 4; c++) f[q][c] = (xc + c < J.W) ? dep_ld(J.sub + y * J.sub_pitch + xc + c) : 0.f;
             }
         }
     }
@@ -452,7 +452,7 @@ __device__ __forceinline__ void sub_thresh_poly_body(const SubThreshJob& J, int 
         if (y >= J.H || xc >= J.W) continue;
         if (J.fused) {
             if (vin && full4) {
-                const float4 t4 = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(J.img) + y * J.pitch + xc));
+                const float4 t4 = dep_ld(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(J.img) + y * J.pitch + xc));
                 f[q][0] = t4.x; f[q][1] = t4.y; f[q][2] = t4.z; f[q][3] = t4.w;
             } else {
 #pragma unroll
@@ -468,7 +468,7 @@ __device__ __forceinline__ void sub_thresh_poly_body(const SubThreshJob& J, int 
 #pragma unroll
                 for (int b = 0; b < 6; b++) {
                     const int64_t xx = xc - 1 + b;
-                    row[a][b] = (yy >= 0 && yy < J.H && xx >= 0 && xx < J.W) ? __ldg(J.sub + yy * J.sub_pitch + xx) : 0.f;
+                    row[a][b] = (yy >= 0 && yy < J.H && xx >= 0 && xx < J.W) ? dep_ld(J.sub + yy * J.sub_pitch + xx) : 0.f;
                 }
             }
             const float wy0 = y > 0 ? 1.f : 0.f, wy2 = y + 1 < J.H ? 1.f : 0.f;
@@ -485,11 +485,11 @@ __device__ __forceinline__ void sub_thresh_poly_body(const SubThreshJob& J, int 
             }
         } else {
             if (vsub && full4) {
-                const float4 t4 = __ldg(reinterpret_cast<const float4*>(J.sub + y * J.sub_pitch + xc));
+                const float4 t4 = dep_ld(reinterpret_cast<const float4*>(J.sub + y * J.sub_pitch + xc));
                 f[q][0] = t4.x; f[q][1] = t4.y; f[q][2] = t4.z; f[q][3] = t4.w;
             } else {
 #pragma unroll
-                for (int c = 0; c < 4; c++) f[q][c] = (xc + c < J.W) ? __ldg(J.sub + y * J.sub_pitch + xc + c) : 0.f;
+                for (int c = 0; c < 4; c++) f[q][c] = (xc + c < J.W) ? dep_ld(J.sub + y * J.sub_pitch + xc + c) : 0.f;
             }
         }
     }
@@ -554,7 +554,7 @@ __device__ bool tile_label_body(const TileJob& J, SH& S, int tile) {
         const int64_t y = ty0 + r, wcol = (tx0 >> 5) + wi;
         uint32_t m = 0;
         if (y < J.H && wcol < J.mw) {
-            m = __ldg(J.mask + y * J.mw + wcol);
+            m = dep_ld(J.mask + y * J.mw + wcol);
             const int64_t valid = J.W - 32 * wcol;
             if (valid < 32) m &= valid > 0 ? ((1u << valid) - 1u) : 0u;
         }
@@ -634,7 +634,7 @@ __device__ bool tile_label_body(const TileJob& J, SH& S, int tile) {
         for (int c0 = st; c0 <= en; c0 += 8) {  // 8 loads in flight, summed in column order
             float f[8];
 #pragma unroll
-            for (int u = 0; u < 8; u++) f[u] = c0 + u <= en ? __ldg(row + c0 + u) : 0.f;
+            for (int u = 0; u < 8; u++) f[u] = c0 + u <= en ? dep_ld(row + c0 + u) : 0.f;
 #pragma unroll
             for (int u = 0; u < 8; u++)
                 if (c0 + u <= en) {

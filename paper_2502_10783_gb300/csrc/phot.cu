@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(P_THREADS) k_centroid(CenJob J) {
                     for (int m = 0; m < NC; m++) {
                         const int64_t i = ia + dii[m], j = ja + dji[m];
                         const bool ok = (lane + 32 * m < nbox) && i >= 0 && i < J.H && j >= 0 && j < J.W;
-                        cache[m] = ok ? __ldg(J.sub + i * J.pitch + j) : 0.f;
+                        cache[m] = ok ? dep_ld(J.sub + i * J.pitch + j) : 0.f;
                         valid |= (uint32_t)ok << m;
                     }
                     cax = ax;
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(P_THREADS) k_centroid(CenJob J) {
                     const float d2 = fmaf(dx, dx, dy * dy);
                     const int64_t i = ia + di, j = ja + dj;
                     if (d2 < rad2 && i >= 0 && i < J.H && j >= 0 && j < J.W) {
-                        const float w = __expf(-d2 * inv2s2) * __ldg(J.sub + i * J.pitch + j);
+                        const float w = __expf(-d2 * inv2s2) * dep_ld(J.sub + i * J.pitch + j);
                         s0 += w;
                         s1 = fmaf(w, dx, s1);
                         s2 = fmaf(w, dy, s2);
@@ -170,7 +170,7 @@ __device__ __forceinline__ void centroid_rows_body(const CenJob& J, int vb, int 
                 for (int c = 0; c < CB; c++) {
                     const int64_t j = ja + (c - R);
                     const bool ok = rowlane && c < box && i >= 0 && i < J.H && j >= 0 && j < J.W;
-                    row[c] = ok ? __ldg(J.sub + i * J.pitch + j) : 0.f;
+                    row[c] = ok ? dep_ld(J.sub + i * J.pitch + j) : 0.f;
                 }
                 cax = ax;
                 cay = ay;
@@ -676,7 +676,7 @@ __device__ __forceinline__ void aperture_body(const PhotJob& J, int vb, int nvb)
                 const int64_t i = ia + di, j = ja + dj;
                 if (i < 0 || i >= J.H || j < 0 || j >= J.W) continue;
             }
-            const float v = __ldg(p0 + di * J.pitch + dj);
+            const float v = dep_ld(p0 + di * J.pitch + dj);
             const float w = t < ni ? 1.0f
                             : (tab ? grid_pixel_area(ktab[wib], R1, di, dj, ox, oy)
                                    : circle_pixel_area(ox - (float)dj, oy - (float)di, J.r_ap));
@@ -696,7 +696,7 @@ __device__ __forceinline__ void aperture_body(const PhotJob& J, int vb, int nvb)
             int first = 0;
             if (inside) {
 #pragma unroll 4
-                for (int t = lane; t < nall; t += 32) buf[t] = __ldg(p0 + (off_di(l_ann[t]) * pitch32 + off_dj(l_ann[t])));
+                for (int t = lane; t < nall; t += 32) buf[t] = dep_ld(p0 + (off_di(l_ann[t]) * pitch32 + off_dj(l_ann[t])));
                 na = first = nall;
             }
             for (int base = first; base < nac; base += 32 * NCH) {
@@ -710,7 +710,7 @@ __device__ __forceinline__ void aperture_body(const PhotJob& J, int vb, int nvb)
                     const int64_t i = ia + di, j = ja + dj;
                     take[c] = t < nac && (inside || (i >= 0 && i < J.H && j >= 0 && j < J.W)) &&
                               in_annulus((float)dj - ox, (float)di - oy, i, j, x, y, rin2, rout2, rin2d, rout2d);
-                    v[c] = take[c] ? __ldg(p0 + di * J.pitch + dj) : 0.f;
+                    v[c] = take[c] ? dep_ld(p0 + di * J.pitch + dj) : 0.f;
                 }
 #pragma unroll
                 for (int c = 0; c < NCH; c++) {

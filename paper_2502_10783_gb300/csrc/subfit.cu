@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(256) k_sub_conv(SubFitJob J, int parts) {
     const bool inb = x0 >= 0 && y0 >= 0 && x0 + WS <= J.W && y0 + WS <= J.H;
     for (int t = threadIdx.x; t < WS * WS; t += 256) {
         const int r = t / WS, q = t - r * WS;
-        Rw[t] = inb ? (double)__ldg(J.R + (int64_t)(y0 + r) * J.pitch + (x0 + q)) : 0.0;
+        Rw[t] = inb ? (double)dep_ld(J.R + (int64_t)(y0 + r) * J.pitch + (x0 + q)) : 0.0;
     }
     __syncthreads();
     // rows: T[f][r][q] = sum_u h_f(u) R(x - u, row r), x = footprint column q
@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(256) k_sub_gram(SubFitJob J, int parts) {
     for (int p = threadIdx.x; p < nfp; p += 256) {
         const int pr = p / FW, pq = p - pr * FW;
         const int x = cx - J.fh + pq, y = cy - J.fh + pr;
-        Is[p] = inb ? (double)__ldg(J.I + (int64_t)y * J.pitch + x) : 0.0;
+        Is[p] = inb ? (double)dep_ld(J.I + (int64_t)y * J.pitch + x) : 0.0;
         if (ng) {
             double tb[64];
             sub_terms_dev((double)x, (double)y, J.W, J.H, J.bord, tb);
