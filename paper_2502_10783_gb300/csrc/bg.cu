@@ -55,6 +55,8 @@ struct MeshShared {
     long long ks_i[2];   // running sums of the kept set (clip loop, warp 0 lane 0)
     df ks_o[2];
     df st[3];            // median, mean, sigma of the kept set
+    long long r1_i[2];   // sums of read 1
+    df r1_o[2];
     float bc_f[8];
     int bc_i[BI_COUNT];
 };
@@ -735,10 +737,10 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
         if (lane == 0) { S.redf[warp] = vmin; S.redf[MS_WARPS + warp] = vmax; }
     }
     __syncthreads();
-    // sums of read 1 (lane 0 of warp 0): their mean and sigma re-place a missed window,
-    // and only then pay for FP64 arithmetic on the serial path (10 K cycles a mesh)
-    long long r1_i1 = 0, r1_i2 = 0;
-    df r1_o1{0.f, 0.f}, r1_o2{0.f, 0.f};
+    // sums of read 1: their mean and sigma re-place a missed window, and only then pay
+    // for FP64 arithmetic on the serial path (10 K cycles a mesh).  They wait in shared
+    // memory: ten registers held through the window search cost a 2048 x 2048 frame of
+    // 64 px meshes 6 us (65 us with the FP64 in every mesh, 71 in registers, 58 here)
     const int e_r1 = e;
     const float c_r1 = cstar;
     if (warp == 0) {
@@ -752,7 +754,7 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
             S.bc_i[BI_N0] = c[0];
             S.bc_f[2] = a;
             S.bc_f[3] = b;
-            r1_i1 = i1; r1_i2 = i2; r1_o1 = o1; r1_o2 = o2;
+            S.r1_i[0] = i1; S.r1_i[1] = i2; S.r1_o[0] = o1; S.r1_o[1] = o2;
         }
     }
     __syncthreads();
@@ -796,8 +798,8 @@ __device__ __forceinline__ void mesh_stats_body(const MeshJob& J, const int mesh
                 const int ends = (int)(S.hbuf[0] + S.hbuf[MS_NB + 1]);
                 if (round < 2 && ((round == 0 && S.bc_i[BI_SBAD]) || b50 == 0 || b50 == MS_NB + 1 || ends > n0 / 8)) {
                     const double unit0 = ldexp(1.0, e_r1 - MS_SCALE_BITS);
-                    const double m1 = ((double)r1_i1 * unit0 + df_to_d(r1_o1)) / n0;
-                    const double var = ((double)r1_i2 * unit0 * unit0 + df_to_d(r1_o2)) / n0 - m1 * m1;
+                    const double m1 = ((double)S.r1_i[0] * unit0 + df_to_d(S.r1_o[0])) / n0;
+                    const double var = ((double)S.r1_i[1] * unit0 * unit0 + df_to_d(S.r1_o[1])) / n0 - m1 * m1;
                     const float mu0 = (float)((double)c_r1 + m1), sd0 = (float)sqrt(fmax(var, 0.0));
                     float span = fmaxf(8.0f * sd0, (vmax - vmin) * 1e-6f);
                     span = fmaxf(span, fabsf(mu0) * 1e-6f + 1e-30f);
