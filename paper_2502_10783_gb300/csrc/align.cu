@@ -292,8 +292,9 @@ __global__ void __launch_bounds__(T) k_aff_sum2(AffPts P, double* __restrict__ p
 // double-float start, so that the ~250 instructions of a start are paid once per
 // group and not once per segment (they were half of the instructions of a segment's
 // 128 pixels).  4096 x 4096: 71 -> 54 us.
-constexpr int RP_GRP = 8;
+constexpr int RP_GRP = 8;     // segments a warp takes at most
 constexpr int RP_SEG = 128;   // output pixels per warp task (4 per lane)
+constexpr int RP_WARPS = 16;  // warps an SM below which a group is halved
 
 // df x exact float (|n| < 2^24): the product to ~2^-46 relative
 __device__ __forceinline__ df df_mul_exact(df m, float n) {
@@ -347,7 +348,7 @@ __device__ __forceinline__ float rp_careful(const float* src, int64_t pitch, int
 __global__ void __launch_bounds__(AL_T) k_reproject(const float* src, int64_t W, int64_t H,
                                                     int64_t pitch, const double* Minv, int64_t Wo,
                                                     int64_t Ho, float fill, float* __restrict__ out,
-                                                    int64_t opitch, bool vout) {
+                                                    int64_t opitch, bool vout, int grp) {
     dep_begin();
     // the transform as double-floats, converted once per block: FP64 work on
     // this GPU's narrow FP64 pipe stays off the per-pixel and per-segment path
@@ -376,12 +377,12 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* src, int64_t W,
     const int64_t warps = (int64_t)gridDim.x * (AL_T / 32);
     const float lim = 1073741824.f;   // 2^30: positions beyond are outside any frame
     const int Wi = (int)W, Hi = (int)H;
-    for (int64_t t0 = ((int64_t)blockIdx.x * (AL_T / 32) + (threadIdx.x >> 5)) * RP_GRP; t0 < tasks;
-         t0 += warps * RP_GRP) {
+    for (int64_t t0 = ((int64_t)blockIdx.x * (AL_T / 32) + (threadIdx.x >> 5)) * grp; t0 < tasks;
+         t0 += warps * grp) {
         // lane l: segment t0 + l's row, first column and source position
         int mi = 0, mj = 0, mbx = 0, mby = 0, mok = 0;
         float mfx = 0.f, mfy = 0.f;
-        if (lane < RP_GRP && t0 + lane < tasks) {
+        if (lane < grp && t0 + lane < tasks) {
             const int64_t i = (t0 + lane) / segs, j0 = (t0 + lane - i * segs) * RP_SEG;
             // first source position of the segment, Minv (j0, i, 1), in double-float
             const float fj = (float)(int)j0, fi = (float)(int)i;   // exact: Wo, Ho < 2^24
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* src, int64_t W,
             mi = (int)i; mj = (int)j0; mbx = ibx; mby = iby; mfx = fbx; mfy = fby;
             mok = (base_ok ? 1 : 0) | (interior ? 2 : 0);
         }
-        const int nseg = (int)min((int64_t)RP_GRP, tasks - t0);
+        const int nseg = (int)min((int64_t)grp, tasks - t0);
         for (int g = 0; g < nseg; g++) {
             const int64_t i = __shfl_sync(0xffffffffu, mi, g), j0 = __shfl_sync(0xffffffffu, mj, g);
             const int ibx = __shfl_sync(0xffffffffu, mbx, g), iby = __shfl_sync(0xffffffffu, mby, g);
@@ -533,7 +534,12 @@ int ipp_launch_reproject(const float* src, int64_t W, int64_t H, int64_t pitch, 
                          int64_t Ho, float fill, float* out, int64_t opitch, cudaStream_t s) {
     const bool vout = (opitch % 4 == 0) && (((uintptr_t)out & 15) == 0);
     const int64_t tasks = ((Wo + RP_SEG - 1) / RP_SEG) * Ho;
-    ipp_launch_dep(k_reproject, dim3(al_grid(AL_T / 32 * RP_GRP, tasks, 8)), AL_T, 0, s, src, W, H, pitch, Minv, Wo, Ho, fill, out, opitch,
-                                                                        vout);
+    // as many segments a warp (1, 2, 4 or 8) as leave RP_WARPS warps an SM.  517 x 389: 9.4
+    // us with eight, 3.9 with one; 1024 x 1024: 9.6, 7.8, and 6.6 with two; 2048 x 2048:
+    // 15.4 and 21.3
+    int grp = RP_GRP;
+    while (grp > 1 && tasks < (int64_t)RP_WARPS * ipp_sm_count() * grp) grp >>= 1;
+    ipp_launch_dep(k_reproject, dim3(al_grid(AL_T / 32 * grp, tasks, 8)), AL_T, 0, s, src, W, H, pitch, Minv, Wo, Ho,
+                   fill, out, opitch, vout, grp);
     return ipp_check_launch("k_reproject");
 }
