@@ -698,12 +698,10 @@ static int launch_fit(const FitJob& J, cudaStream_t s) {
 // shorter.  G is taken while N G stays within 1.25 x the lanes resident at G
 // (measured on 152 SMs, 15 x 15 stamps: G = 4 up to ~12,000 stamps, G = 2 up
 // to ~24,000, G = 1 beyond).
-// G fixes the order of a stamp's sums, so the line does not move with the resident
-// warps of the present kernel: it counts eight warps at most.
 static int fit_lanes_per_stamp(const FitJob& J) {
     const int64_t sms = sm_count();
     for (int G = 4; G > 1; G >>= 1)
-        if (J.N * G * 4 <= sms * std::min(8, fit_max_warps(J.S, G)) * 32 * 5) return G;
+        if (J.N * G * 4 <= sms * fit_max_warps(J.S, G) * 32 * 5) return G;
     return 1;
 }
 
