@@ -461,11 +461,8 @@ __global__ void __launch_bounds__(AL_T) k_reproject(const float* src, int64_t W,
 using namespace ipp;
 
 static unsigned al_grid(int64_t units_per_block_task, int64_t tasks, int per_sm) {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t need = (tasks + units_per_block_task - 1) / units_per_block_task;
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)(sms > 0 ? sms : 152) * per_sm));
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)ipp_sm_count() * per_sm));
 }
 
 static WcsDev to_dev(const ipp_wcs& w) {

@@ -161,9 +161,11 @@ IPP_D int frame_of(const int* bs, int nf, int b) {
 // take their places meanwhile, so that a small frame's 14 launches do not each pay
 // the drain and the start of a grid.  Larger grids, whose waiting successors would
 // hold places that other streams' kernels could use, leave that to their end.
+constexpr unsigned DEP_EARLY = 608;   // blocks: four for each of this part's 152 SMs
+
 IPP_D void dep_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (gridDim.x * gridDim.y <= 608u) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (gridDim.x * gridDim.y <= DEP_EARLY) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // Loads of a kernel that starts with dep_begin(), whose blocks are resident while the

@@ -826,13 +826,6 @@ __global__ void __launch_bounds__(DB_T) k_deblend_write(DeblendJob J) {
 
 using namespace ipp;
 
-static int db_sms() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 132;
-}
-
 int ipp_launch_deblend(const DeblendJob& J, cudaStream_t s) {
     if (cudaMemsetAsync(J.out, 0, sizeof(int32_t) * (size_t)(J.W * J.H), s) != cudaSuccess)
         return ipp_check_launch("deblend memset");
@@ -846,11 +839,11 @@ int ipp_launch_deblend(const DeblendJob& J, cudaStream_t s) {
     int per = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_deblend, DB_T, DB_DYN_BYTES) != cudaSuccess || per < 1)
         per = 1;
-    k_deblend<<<db_sms() * per, DB_T, DB_DYN_BYTES, s>>>(J);
+    k_deblend<<<ipp_sm_count() * per, DB_T, DB_DYN_BYTES, s>>>(J);
     if (int e = ipp_check_launch("k_deblend")) return e;
     k_deblend_scan<<<1, 1024, 0, s>>>(J.n_src_dev, J.max_src, J.ws.nobj, J.ws.offs, J.n_out_dev);
     if (int e = ipp_check_launch("k_deblend_scan")) return e;
-    k_deblend_write<<<db_sms() * 8, DB_T, 0, s>>>(J);
+    k_deblend_write<<<ipp_sm_count() * 8, DB_T, 0, s>>>(J);
     return ipp_check_launch("k_deblend_write");
 }
 

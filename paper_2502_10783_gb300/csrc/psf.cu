@@ -660,13 +660,6 @@ __global__ void __launch_bounds__(256) k_psf_adj(const float* __restrict__ param
 
 using namespace ipp;
 
-static int sm_count() {
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms > 0 ? sms : 132;
-}
-
 static size_t fit_warp_bytes(int S, int G) { return (size_t)S * S * fit_pitch(G) * sizeof(float); }
 static int fit_max_warps(int S, int G) {   // the kernel's static shared memory is 8 bytes
     return (int)std::min<size_t>(FL_MAX_WARPS, (size_t)(227 * 1024 - 64) / fit_warp_bytes(S, G));
@@ -681,8 +674,8 @@ static int launch_fit(const FitJob& J, cudaStream_t s) {
     // smaller the idle tail.  One block per SM, as many warps as its shared
     // memory holds.
     const int wmax = fit_max_warps(J.S, G);
-    const int64_t warps = std::min<int64_t>((int64_t)sm_count() * wmax, (J.N + 32 / G - 1) / (32 / G));
-    const int64_t blocks = std::min<int64_t>(sm_count(), warps);
+    const int64_t warps = std::min<int64_t>((int64_t)ipp_sm_count() * wmax, (J.N + 32 / G - 1) / (32 / G));
+    const int64_t blocks = std::min<int64_t>(ipp_sm_count(), warps);
     const int wpb = (int)((warps + blocks - 1) / blocks);
     const size_t smem = per_warp * wpb;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -699,7 +692,7 @@ static int launch_fit(const FitJob& J, cudaStream_t s) {
 // (measured on 152 SMs, 15 x 15 stamps: G = 4 up to ~12,000 stamps, G = 2 up
 // to ~24,000, G = 1 beyond).
 static int fit_lanes_per_stamp(const FitJob& J) {
-    const int64_t sms = sm_count();
+    const int64_t sms = ipp_sm_count();
     for (int G = 4; G > 1; G >>= 1)
         if (J.N * G * 4 <= sms * fit_max_warps(J.S, G) * 32 * 5) return G;
     return 1;
@@ -729,7 +722,7 @@ template <class Fn>
 static void launch_psf_lanes(int64_t N, int S, Fn&& go) {
     const int L = S <= 6 ? 8 : 32;
     const int64_t need = (N + 256 / L - 1) / (256 / L);
-    go(L, (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)sm_count() * 32)));
+    go(L, (unsigned)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)ipp_sm_count() * 32)));
 }
 
 int ipp_launch_psf_fwd(const float* params, int64_t N, int S, int model, float beta, float* out, cudaStream_t s) {

@@ -965,13 +965,14 @@ SubDims sub_dims(int hw, int fh, int nk, const int32_t* deg, int sord, int bord)
 }
 
 // Blocks a candidate of the FP64-bound kernels, one block an SM: the cut whose
-// waves of 152 / parts candidates take the least time (100 candidates: one part
+// waves take the least time (100 candidates: one part
 // fills 100 SMs once, three fill 152 twice with a third of the work each).
 int sub_parts(int max_c) {
+    const int64_t sms = ipp_sm_count();
     int best = 1;
     double cost = 1e30;
     for (int p = 1; p <= 6; p++) {
-        const double t = (double)(((int64_t)max_c * p + 151) / 152) / p;
+        const double t = (double)cdiv((int64_t)max_c * p, sms) / p;
         if (t < cost * 0.95) { cost = t; best = p; }
     }
     return best;
@@ -1027,7 +1028,7 @@ int ipp_launch_sub_stamps(const float* I, const float* R, int64_t W, int64_t H, 
     const int64_t nreg = (int64_t)nsx * nsy, npix = ((W + nsx - 1) / nsx) * ((H + nsy - 1) / nsy);
     int nc = 1;
     while (nc < SS_NC && (npix > (int64_t)nc * SS_SLICE ||
-                          (nreg * nc * 2 <= 304 && npix >= (int64_t)nc * 2 * 8 * SS_T)))
+                          (nreg * nc * 2 <= 2 * ipp_sm_count() && npix >= (int64_t)nc * 2 * 8 * SS_T)))
         nc *= 2;
     const int slice = (int)std::min<int64_t>(SS_SLICE, npix / nc + 1);
     auto fn = k_sub_stamps;
