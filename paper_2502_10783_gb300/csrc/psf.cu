@@ -129,8 +129,8 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 //       stages each new stamp in shared memory (pixel k of slot s at
 //       k fit_pitch(G) + s) and computes its default starting point together;
 //   (2) slots with a fit in progress solve their damped normal equations (FP64); one
-//       whose step promises little is put on hold until its convergence test, a
-//       second solve, can be made for several slots at once;
+//       whose step promises little takes its convergence test, a second solve -- at
+//       G = 1 it is put on hold until that can be made for several slots at once;
 //   (3) every slot with a point to try evaluates chi^2, J'WJ and J'Wr there,
 //       each lane of the slot over every G-th stamp row, and the slot's lanes
 //       add their sums with shuffles;
@@ -155,11 +155,12 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 // with the forms of eval_lane and border_pair below.
 constexpr int FL_MAX_WARPS = 8;
 
-// Slots on hold for which the undamped system is solved (fewer when nothing else is
-// left to do in the warp).  A solve costs the warp the same FP64 time for one lane
-// as for 32, and with 32 fits a warp one of them converges in almost every round:
-// solved at once, the second solve doubled the FP64 work; waiting costs a slot a
-// round or two.
+// G = 1: slots on hold for which the undamped system is solved (fewer when nothing else is
+// left to do in the warp, or no stamp waits for a slot).  A solve costs the warp the same
+// FP64 time for one lane as for 32, and with 32 fits a warp one of them converges in
+// almost every round: solved at once, the second solve doubled the FP64 work; waiting
+// costs a slot a round or two, which only a waiting stamp can make good: 50,000 stamps of
+// 11 x 11, Gaussian, 2510 us solved at once, 2600 held to the end, 2450 so.
 constexpr int HOLD_MIN = 4;
 
 // Base-2 logarithm, exponential and quotient of the hardware without the steps that
@@ -427,52 +428,90 @@ __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t
             for (int a = 0; a < 7; a++) pt[a] = p[a];
             try_pt = true;
         }
-        // pass 0: the damped step of every slot with a fit in progress; pass 1: the
-        // undamped system of the slots on hold.  One copy of the solve's code.
+        // A fit has converged when the Gauss-Newton decrease g'H^-1 g is below what the
+        // distance to the optimum (1e-10 chi^2) and the model's FP32 rounding
+        // (1e-12 sum w P^2) allow; the damped step's decrease never exceeds it, so the
+        // undamped system is solved only when that one is small.
+        if constexpr (G > 1) {
+            // few fits a warp: both systems at once (with the form below, 8000 stamps of
+            // 15 x 15 took 1457 us, 1397 so)
+            if (st >= 0 && !fresh) {
+                double x[7];
+                if (!solve7(H, g, lam, x)) {
+                    lam *= 10.0;
+                    nsing++;
+                    it++;
+                    if (lam > 1e10) fl = IPP_FLAG_FIT_MAXITER;
+                } else {
+                    const double thr = 1e-10 * widen(chi2) + 1e-12 * widen(sm2);
+                    double dec = 0.0;
+#pragma unroll
+                    for (int a = 0; a < 7; a++) dec = fma(widen(g[a]), x[a], dec);
+                    if (dec <= thr) {
+                        double u[7];
+                        if (solve7(H, g, 0.0, u)) {
+                            double dgn = 0.0;
+#pragma unroll
+                            for (int a = 0; a < 7; a++) dgn = fma(widen(g[a]), u[a], dgn);
+                            if (dgn <= thr) fl = 0;   // stopped at p
+                        }
+                    }
+#pragma unroll
+                    for (int a = 0; a < 7; a++) pt[a] = narrow(widen(p[a]) + x[a]);
+                    if (fl == 0) {
+                    } else if (!(pt[4] > 0.05f) || !(pt[5] > 0.05f)) {
+                        lam *= 10.0;
+                        it++;
+                        if (lam > 1e10) fl = 0;
+                    } else {
+                        try_pt = true;
+                    }
+                }
+            }
+        } else {
+            // pass 0: the damped step of every slot with a fit in progress; pass 1: the
+            // undamped system of the slots on hold.  One copy of the solve's code.
 #pragma unroll 1
-        for (int pass = 0; pass < 2; pass++) {
-            bool run = st >= 0 && !fresh && !hold;
-            if (pass == 1) {
-                const unsigned held = __ballot_sync(FULL, hold) & HEADS;
-                const bool due = __popc(held) >= HOLD_MIN / G || !__any_sync(FULL, try_pt);
-                run = hold && due;
-            }
-            if (!__any_sync(FULL, run)) continue;
-            if (!run) continue;
-            double x[7];
-            const bool ok = solve7(H, g, pass == 0 ? lam : 0.0, x);
-            if (!ok && pass == 0) {
-                lam *= 10.0;
-                nsing++;
-                it++;
-                if (lam > 1e10) fl = IPP_FLAG_FIT_MAXITER;
-                continue;
-            }
-            // converged when the Gauss-Newton decrease g'H^-1 g is below what the
-            // distance to the optimum (1e-10 chi^2) and the model's FP32 rounding
-            // (1e-12 sum w P^2) allow; the damped step's decrease never exceeds
-            // it, so the undamped system is solved only when that one is small
-            const double thr = 1e-10 * widen(chi2) + 1e-12 * widen(sm2);
-            double dec = 0.0;
+            for (int pass = 0; pass < 2; pass++) {
+                bool run = st >= 0 && !fresh && !hold;
+                if (pass == 1) {
+                    const int held = __popc(__ballot_sync(FULL, hold));
+                    const bool due = held >= HOLD_MIN || drained || !__any_sync(FULL, try_pt);
+                    run = hold && due;
+                }
+                if (!__any_sync(FULL, run)) continue;
+                if (!run) continue;
+                double x[7];
+                const bool ok = solve7(H, g, pass == 0 ? lam : 0.0, x);
+                if (!ok && pass == 0) {
+                    lam *= 10.0;
+                    nsing++;
+                    it++;
+                    if (lam > 1e10) fl = IPP_FLAG_FIT_MAXITER;
+                    continue;
+                }
+                const double thr = 1e-10 * widen(chi2) + 1e-12 * widen(sm2);
+                double dec = 0.0;
 #pragma unroll
-            for (int a = 0; a < 7; a++) dec = fma(widen(g[a]), x[a], dec);
-            const bool small = ok && dec <= thr;
-            if (pass == 0) {
+                for (int a = 0; a < 7; a++) dec = fma(widen(g[a]), x[a], dec);
+                const bool small = ok && dec <= thr;
+                if (pass == 0) {
 #pragma unroll
-                for (int a = 0; a < 7; a++) pt[a] = narrow(widen(p[a]) + x[a]);
-                hold = small;
-                if (hold) continue;
-            } else {
-                hold = false;
-                if (small) fl = 0;   // stopped at p
-            }
-            if (fl == 0) {
-            } else if (!(pt[4] > 0.05f) || !(pt[5] > 0.05f)) {
-                lam *= 10.0;
-                it++;
-                if (lam > 1e10) fl = 0;
-            } else {
-                try_pt = true;
+                    for (int a = 0; a < 7; a++) pt[a] = narrow(widen(p[a]) + x[a]);
+                    hold = small;
+                    if (hold) continue;
+                } else {
+                    hold = false;
+                    if (small) fl = 0;   // stopped at p
+                }
+                if (fl == 0) {
+                } else if (!(pt[4] > 0.05f) || !(pt[5] > 0.05f)) {
+                    lam *= 10.0;
+                    it++;
+                    if (lam > 1e10) fl = 0;
+                } else {
+                    try_pt = true;
+                }
             }
         }
         float Ht[28], gt[7], c2t = 0.f, s2t = 0.f;
