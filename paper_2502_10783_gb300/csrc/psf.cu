@@ -163,22 +163,12 @@ constexpr int FL_MAX_WARPS = 8;
 // 11 x 11, Gaussian, 2510 us solved at once, 2600 held to the end, 2450 so.
 constexpr int HOLD_MIN = 4;
 
-// Base-2 logarithm, exponential and quotient of the hardware without the steps that
-// extend them to subnormals: 1 + q >= 1 has none, and a profile value or derivative
-// below 2^-126 adds nothing to the sums.
+// Base-2 logarithm of the hardware without the steps for subnormal arguments: 1 + q >= 1
+// has none.  (The exponential and the quotient keep theirs: a profile far out is part of a
+// fit whose star lies off its stamp.)
 __device__ __forceinline__ float lg2_fast(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float ex2_fast(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float div_fast(float a, float b) {
-    float y;
-    asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
     return y;
 }
 
@@ -222,14 +212,14 @@ __device__ __forceinline__ float eval_lane(const float* __restrict__ col, const 
             const float q = fmaf(u, a, v * b);
             float A1, P, T;
             if (MODEL == IPP_PSF_GAUSS) {
-                A1 = A0 * ex2_fast(-0.72134752f * q);  // exp(-q/2)
+                A1 = A0 * exp2f(-0.72134752f * q);  // exp(-q/2)
                 P = F * A1;
                 T = -P;
             } else {
                 const float base = 1.0f + q;
-                A1 = A0 * ex2_fast(-beta * lg2_fast(base));
+                A1 = A0 * exp2f(-beta * lg2_fast(base));
                 P = F * A1;
-                T = div_fast(tq * P, base);
+                T = __fdividef(tq * P, base);
             }
             const float wk = WEIGHTED ? __ldg(wts + i * S + j) : 1.0f;
             const float r = row[j * PITCH] - (P + sky);
