@@ -110,14 +110,6 @@ __device__ __forceinline__ bool mesh_value_at(const GG& G, int r, int c, float* 
     return !(G.mask && G.mask[yy * G.W + xx]) && isfinite(x);
 }
 
-// Calls f(v) for every usable value of the mesh that this thread owns (raw frames
-// whose rows and maps are aligned: mesh_for_each_u16 above).  Vector
-// path: float4 quads of the mesh's frame region, quad e4 = threadIdx.x + k *
-// MS_THREADS; scalar path: element e = threadIdx.x + k * MS_THREADS of the
-// mw x mh slots (row e / mw, column e % mw).  A chunk of loads is issued before
-// any is used: addresses are clamped into the mesh and slots beyond it are
-// skipped afterwards.  Every call forms the values with the same arithmetic, so
-// re-reads see identical values.
 // The quads of a raw frame: 8 bytes of the frame and 16 of the inverse flat (and of
 // the bias map) a load, where the scalar path takes four loads of each and their
 // addresses.  4096 x 4096 raw frame, 128 px meshes: k_mesh_stats 206 -> 120 us.
@@ -159,6 +151,13 @@ __device__ __forceinline__ void mesh_for_each_u16(const MeshGeom& G, F& f) {
     }
 }
 
+// Calls f(v) for every usable value of the mesh that this thread owns.  Vector path
+// (that of raw frames with aligned rows and maps: mesh_for_each_u16 above): float4 quads
+// of the mesh's frame region, quad e4 = threadIdx.x + k * MS_THREADS; scalar path:
+// element e = threadIdx.x + k * MS_THREADS of the mw x mh slots (row e / mw, column
+// e % mw).  A chunk of loads is issued before any is used: addresses are clamped into
+// the mesh and slots beyond it are skipped afterwards.  Every call forms the values with
+// the same arithmetic, so re-reads see identical values.
 template <int T = MS_THREADS, class GG, class F>
 __device__ __forceinline__ void mesh_for_each(const GG& G, F&& f) {
     if (GG::kind != MK_U16 && G.vec) {
