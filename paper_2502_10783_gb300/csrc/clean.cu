@@ -283,6 +283,15 @@ __device__ __forceinline__ void kahan_acc(float& s, float& c, float v) {
     s = t;
 }
 
+// 1 / x for x of about 1 and above, by the hardware's reciprocal without the steps for
+// subnormal arguments and results: x = 1 + q has none below 2^126, where a profile is 0
+// either way.  The product with a peak keeps subnormal values.
+__device__ __forceinline__ float rcp_fast(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 template <bool UNIT>
 __global__ void __launch_bounds__(CL_T) k_clean_pairs(const int32_t* n_dev, int32_t max_obj, CleanWs ws, int64_t W,
                                                       float beta) {
@@ -329,7 +338,7 @@ __global__ void __launch_bounds__(CL_T) k_clean_pairs(const int32_t* n_dev, int3
             const float dx = (px - a.x) - a.w, dy = (py - a.y) - e.w;
             // r^2 / a^2 = dx (y2' dx - 2 xy' dy) + x2' dy^2
             const float q = fmaf(dx, fmaf(e.x, dx, e.y * dy), e.z * dy * dy);
-            const float mv = UNIT ? __fdividef(a.z, 1.0f + q) : a.z * expf(-beta * log1pf(q));
+            const float mv = UNIT ? a.z * rcp_fast(1.0f + q) : a.z * expf(-beta * log1pf(q));
             kahan_acc(sum, comp, mv);
             if (mv >= best) {                              // ties to the smaller label (rare)
                 const int lj = sb[t];
