@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(T) k_aff_sum2(AffPts P, double* __restrict__ p
 }
 
 // ---- bilinear reprojection ---------------------------------------------------------
-// A warp takes RP_GRP consecutive segments: its first lanes each form one segment's
+// A warp takes up to RP_GRP consecutive segments: its first lanes each form one segment's
 // double-float start, so that the ~250 instructions of a start are paid once per
 // group and not once per segment (they were half of the instructions of a segment's
 // 128 pixels).  4096 x 4096: 71 -> 54 us.

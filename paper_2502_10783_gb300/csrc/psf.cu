@@ -151,8 +151,9 @@ __device__ __forceinline__ bool solve7(const float Hf[28], const float gf[7], do
 // that the stamps' tiles leave room for, so at G = 1 a tile has no padding column
 // (15 x 15 stamps: 28.1 KB, eight warps an SM; 29 KB and seven before): a row, one
 // pixel of 32 stamps, is read without conflicts, and only the staging stores, one
-// stamp's column, meet in one bank.  200,000 stamps of 15 x 15: 15.3 -> 12.2 ms
-// with the forms of eval_lane and border_pair below.
+// stamp's column, meet in one bank (the registers, 248 and more a thread, hold eight
+// warps as well).  200,000 stamps of 15 x 15: 15.3 -> 12.7 ms with the forms of eval_lane
+// and border_pair below.
 constexpr int FL_MAX_WARPS = 8;
 
 // G = 1: slots on hold for which the undamped system is solved (fewer when nothing else is
@@ -563,9 +564,9 @@ __global__ void __launch_bounds__(32 * FL_MAX_WARPS) k_psf_fit(FitJob J, int64_t
 // once per stamp instead of once per pixel, and a lane walks its pixels (lane,
 // lane + L, ...) by adding L in (row, column) form, without a division.  Both are
 // bound by issue slots (the logarithm and exponential of a pixel), then by the
-// 4 bytes a pixel of DRAM.  50,000 Moffat stamps of 15 x 15: forward 71 -> 35 us
+// 4 bytes a pixel of DRAM.  50,000 Moffat stamps of 15 x 15: forward 72 -> 35 us
 // (one thread per pixel, sincos and 64-bit divisions in each, before), adjoint
-// 87 -> 48 us.
+// 82 -> 55 us.
 struct PsfStamp {
     float x0, y0, F, sky, sx, sy, isx, isy, c, s, amp;   // amp: dm/dF at the centre
 };
@@ -719,7 +720,9 @@ static int launch_fit(const FitJob& J, cudaStream_t s) {
 // stamp, so that the batch still spreads over the lanes and each round is
 // shorter.  G is taken while N G stays within 1.25 x the lanes resident at G
 // (measured on 152 SMs, 15 x 15 stamps: G = 4 up to ~12,000 stamps, G = 2 up
-// to ~24,000, G = 1 beyond).
+// to ~24,000, G = 1 beyond).  With a count on the device N is the capacity of the arrays:
+// G, and with it the order of a stamp's sums, can differ from a call that is given the
+// same stamps by their number.
 static int fit_lanes_per_stamp(const FitJob& J) {
     const int64_t sms = ipp_sm_count();
     for (int G = 4; G > 1; G >>= 1)
